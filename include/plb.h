@@ -169,7 +169,8 @@ int plb_init(plb_t *h, const double *rho0, const double *u0);
 int plb_init_physical(plb_t *h, const double *rho0, const double *u0);
 
 /* Advances n time steps (two kernels per step: psi pass, then the fused force +
- * collide + stream pass).  Asynchronous; returns launch errors only.  Device-side
+ * collide + stream pass; lattices of up to 2^18 cells take many steps in one launch, with
+ * the same result).  Asynchronous; returns launch errors only.  Device-side
  * faults of the method (psi domain, non-finite density) are recorded in a device flag
  * and reported by plb_status / plb_moments / plb_reduce. */
 int plb_step(plb_t *h, int n);
@@ -180,7 +181,8 @@ int plb_step(plb_t *h, int n);
 int plb_step_timed(plb_t *h, int n, double ms[2]);
 
 /* Synchronises the stream and returns PLB_EPSI_DOMAIN / PLB_ENONFINITE if a kernel
- * met such a cell since creation or the last plb_init, else PLB_OK. */
+ * met such a cell since creation or the last plb_init, PLB_ETIMEOUT if a bounded wait inside
+ * a step gave up (the populations are then undefined until the next plb_init), else PLB_OK. */
 int plb_status(plb_t *h);
 
 /* Number of steps since plb_init; -1 for a NULL handle. */

@@ -25,7 +25,7 @@ struct Layout {
     long long psi_elems;
     long long chunk;        // cells per staging chunk
     int max_blocks;         // reduction partial blocks
-    size_t off_pops, off_pops2, off_psi, off_partials, off_out, off_staging, off_flags, total;
+    size_t off_pops, off_pops2, off_psi, off_partials, off_out, off_staging, off_flags, off_counts, total;
 };
 
 // streaming = PLB_STREAM_FUSED adds the second population copy (off_pops2; else off_pops2 = off_pops).
@@ -69,6 +69,9 @@ struct plb_state {
     long long t;
     int odd;
     int view;                  // 1: an instance of a batch (stepped only by plb_batch_step)
+    unsigned *counts;          // step counts of the many-step launch's tiles (NULL: not used)
+    plb::TileArgs tiles;       // its split of the lattice, planned at the first step
+    int tiles_state;           // 0: not planned yet, 1: planned, -1: not for this lattice
     int slab;                  // 1: a z-slab whose first and last planes are ghost planes (plb_slab_*)
     int slab_stage;            // slab: 0 = the next pass is the psi pass, 1 = the collide pass
 };

@@ -11,6 +11,7 @@
 #include "plb_pair.cuh"
 #include "plb_staged.cuh"
 #include "plb_step.cuh"
+#include "plb_tile.cuh"
 
 // L2 prefetch one wave ahead in the FP32 fused pass (1) or not (0).
 #ifndef PLB_L2_PREFETCH
@@ -576,6 +577,104 @@ template <class L, class S> struct Launch {
     }
     static void fused_bgk(const KParams &p, const void *A, void *B, cudaStream_t st) { fused_t<0>(p, A, B, st); }
     static void fused_mrt(const KParams &p, const void *A, void *B, cudaStream_t st) { fused_t<1>(p, A, B, st); }
+    // kernel of the many-step launch for this lattice and collision form (FORM 1: the single pass's)
+    template <int FORM> static const void *tile_kernel(const KParams &p, int mrt) {
+        constexpr int M = FORM && !Store<S>::SHIFT && std::is_same<L, D3Q19>::value ? PLB_FUSED_MOMENT : -1;
+        if constexpr (std::is_same<S, double>::value) {
+            return mrt ? (const void *)&k_tile<L, S, 1, false, -1, 1> : (const void *)&k_tile<L, S, 0, false, -1, 1>;
+        } else {
+            if constexpr (Store<S>::SHIFT) {
+                if (p.stochastic) {
+                    if (p.nx % 2 == 0)
+                        return mrt ? (const void *)&k_tile<L, S, 1, true, M, 2> : (const void *)&k_tile<L, S, 0, true, M, 2>;
+                    return mrt ? (const void *)&k_tile<L, S, 1, true, -1, 1> : (const void *)&k_tile<L, S, 0, true, -1, 1>;
+                }
+            }
+            if (p.nx % 2 == 0)
+                return mrt ? (const void *)&k_tile<L, S, 1, false, M, 2> : (const void *)&k_tile<L, S, 0, false, M, 2>;
+            return mrt ? (const void *)&k_tile<L, S, 1, false, -1, 1> : (const void *)&k_tile<L, S, 0, false, -1, 1>;
+        }
+    }
+    static size_t tile_smem(const KParams &p, const TileArgs &t) {
+        const int w = !std::is_same<S, double>::value && p.nx % 2 == 0 ? 2 : 1;
+        const size_t v = w * sizeof(typename Store<S>::T);
+        return ((size_t)L::Q * v + 4) * t.max_own + (size_t)(w * sizeof(PsiT) + 8) * t.max_region;
+    }
+    // Splits the lattice into tiles: the split with the least cost, which is the work of the fullest SM
+    // (throughput) plus 256 threads' worth for every pass of a block over its cells (latency).
+    // Which lattices: up to 2^18 cells (the staging area then holds the second copy; at 64^3 FP32 the
+    // tiles still win, 10.8 us a step against 14.6), FP64 D3Q19 only to 2^14 (bound by the FP64 pipe, where
+    // the ring's psi is extra work: 24^3 41 us against 47, 32^3 126 against 123).
+    template <int FORM> static bool tile_plan(const KParams &p, int mrt, TileArgs &t) {
+        const void *k = tile_kernel<FORM>(p, mrt);
+        const int w = !std::is_same<S, double>::value && p.nx % 2 == 0 ? 2 : 1;
+        const int nw = p.nx / w, sms = sm_count();
+        if (p.n > (std::is_same<S, double>::value && L::D == 3 ? 1LL << 14 : 1LL << 18)) return false;
+        const size_t most = 200 * 1024;
+        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        long long best = -1;
+        constexpr int ring = L::D == 3 ? 2 : 0;
+        TileArgs c = t;
+        const int unit = w == 2 ? tile_unit<S, 2> : tile_unit<S, 1>, units = tile_units(nw, unit);
+        for (c.gx = 1; c.gx <= 16 && c.gx <= units; ++c.gx) {
+            for (c.gz = 1; c.gz <= 32 && (c.gz == 1 || p.nz / c.gz >= 2); ++c.gz) {
+                for (int per_sm = 1; per_sm <= 3; ++per_sm) {
+                    c.gy = sms * per_sm / (c.gx * c.gz);
+                    if (c.gy > p.ny / 2) c.gy = p.ny / 2;
+                    if (c.gy < 1) c.gy = 1;
+                    const long long tiles = (long long)c.gx * c.gy * c.gz;
+                    if (tiles > kMaxTiles || tiles > (long long)sms * per_sm) continue;
+                    int tw = (units + c.gx - 1) / c.gx * unit + (nw % unit == 1 ? 1 : 0);
+                    tw = units == 1 || tw > nw ? nw : tw;
+                    const int th = (p.ny + c.gy - 1) / c.gy, td = (p.nz + c.gz - 1) / c.gz;
+                    if (tw > 1023 || th > 1023 || td > 1023) continue;
+                    c.max_own = (tw * th * td + 1) & ~1;          // even: 8-byte alignment of what follows
+                    c.max_region = ((tw + 2) * (th + 2) * (td + ring) + 1) & ~1;
+                    const int here = (int)((tiles + sms - 1) / sms);       // blocks on the fullest SM
+                    c.threads = TileThreads<L, S>::per_sm / here / 32 * 32;
+                    if (c.threads > TileThreads<L, S>::most) c.threads = TileThreads<L, S>::most;
+                    const int even = ((c.max_region + 31) / 32) * 32;
+                    if (c.threads > even) c.threads = even < 64 ? 64 : even;
+                    const long long fit = (long long)(227 * 1024) / (long long)(tile_smem(p, c) + 1024);
+                    if (fit < here || tile_smem(p, c) > most) continue;
+                    // a collision in units of psi of a region cell: 2 in FP32 (64^3: 1900 cycles a pass
+                    // for psi, 4400 for the collision), 8 in FP64 (60 and 424 pipe operations)
+                    const int cost = std::is_same<S, double>::value ? 8 : 2;
+                    const long long rounds = (c.max_region + c.threads - 1) / c.threads +
+                                             cost * ((c.max_own + c.threads - 1) / c.threads);
+                    const long long work = here * ((long long)cost * c.max_own + c.max_region) + 256 * rounds;
+                    if (best < 0 || work < best) {
+                        best = work;
+                        t = c;
+                    }
+                }
+            }
+        }
+        if (best < 0) return false;
+        int nb = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, t.threads, tile_smem(p, t)) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        return (long long)nb * sms >= (long long)t.gx * t.gy * t.gz;
+    }
+    template <int FORM> static cudaError_t tile_run(const KParams &p, int mrt, const TileArgs &t, cudaStream_t st) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(t.gx * t.gy * t.gz, 1, 1);
+        cfg.blockDim = dim3(t.threads, 1, 1);
+        cfg.dynamicSmemBytes = tile_smem(p, t);
+        cfg.stream = st;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeCooperative;
+        attr[0].val.cooperative = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        void *args[] = {const_cast<KParams *>(&p), const_cast<TileArgs *>(&t)};
+        return cudaLaunchKernelExC(&cfg, tile_kernel<FORM>(p, mrt), args);
+    }
     static const void *batch_bgk() { return reinterpret_cast<const void *>(&k_batch<L, S, 0>); }
     static const void *batch_mrt() { return reinterpret_cast<const void *>(&k_batch<L, S, 1>); }
     static constexpr Launchers table() {
@@ -583,6 +682,7 @@ template <class L, class S> struct Launch {
                          {&batch_bgk, &batch_mrt}, &rebalance, &wall_fill,
                          {std::is_same<S, double>::value ? nullptr : &fused_bgk,
                           std::is_same<S, double>::value ? nullptr : &fused_mrt},
+                         {&tile_plan<0>, &tile_plan<1>}, {&tile_run<0>, &tile_run<1>},
                          &mass};
     }
 };

@@ -5,7 +5,7 @@
 
 namespace plb {
 
-enum : unsigned { FLAG_PSI_DOMAIN = 1u, FLAG_NONFINITE = 2u, FLAG_BAD_INPUT = 4u };
+enum : unsigned { FLAG_PSI_DOMAIN = 1u, FLAG_NONFINITE = 2u, FLAG_BAD_INPUT = 4u, FLAG_TIMEOUT = 8u };
 // Device flag area of a lattice (64 bytes): word 0 holds the FLAG_* bits; the 8-byte slots
 // at words 2 and 4 hold the first invalid rho0 and u0 index k_init met (all ones if none).
 enum : int { FLAG_SLOT_RHO = 2, FLAG_SLOT_U = 4 };
@@ -92,6 +92,19 @@ struct BatchLaunch {
     unsigned expected;       // blocks the barrier waits for (gridDim.x unless testing a timeout)
 };
 
+// Many steps of a small lattice in one launch: the lattice cut into gx x gy x gz tiles, one per block.
+// Step counts lie kTilePitch words apart: polled counts that share lines cost 2 us a step.
+constexpr int kMaxTiles = 512, kTilePitch = 32, kTileWords = kTilePitch * (1 + kMaxTiles);
+struct TileArgs {
+    void *a, *b;              // population copies: the first step reads a and writes b
+    unsigned *counts;         // [0] a wait gave up, [kTilePitch (1 + tile)] steps the tile has finished
+    int gx, gy, gz;
+    int threads;              // per block
+    int max_own, max_region;  // cells (pairs) of the largest tile, without and with its ring
+    int nsteps;
+    unsigned spin_limit;
+};
+
 struct Launchers {
     void (*init)(const KParams &, void *A, const double *rho0, const double *u0, long long c0, long long cn,
                  cudaStream_t);
@@ -111,6 +124,10 @@ struct Launchers {
     void (*wall_fill)(const KParams &, void *psi, cudaStream_t);
     // single-pass step [BGK, MRT]: reads A (natural layout), pushes into B; NULL for FP64
     void (*fused[2])(const KParams &, const void *A, void *B, cudaStream_t);
+    // t.nsteps steps in one launch [collision form: of the two-pass kernels, of the single pass]: plans the
+    // tiles (t.gx .. t.max_region), false where this lattice is not for it; then launches
+    bool (*tile_plan[2])(const KParams &, int mrt, TileArgs &t);
+    cudaError_t (*tile_run[2])(const KParams &, int mrt, const TileArgs &t, cudaStream_t);
     // total mass of the whole lattice, one partial per block (slot 0 of 4)
     void (*mass)(const KParams &, const void *A, double *partials, int nblocks, cudaStream_t);
 };

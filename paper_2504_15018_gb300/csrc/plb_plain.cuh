@@ -146,12 +146,11 @@ __device__ __forceinline__ double psi(const KParams &p, double rho) {
 }
 
 // Total force density at a cell (Eqs. Shan_Chen_Force, interactionForce, plus the body
-// force) from the padded psi field; pc points at the cell's psi.
+// force) from a psi field of row pitch sy and plane pitch sz; pc points at the cell's psi.
 template <class L, class Pol>
-__device__ __forceinline__ void force(const KParams &p, const double *__restrict__ pc, double F[3]) {
+__device__ __forceinline__ void force(const KParams &p, const double *__restrict__ pc, int sy, int sz, double F[3]) {
     constexpr int D = L::D;
     const PlainPhys &q = p.pl;
-    const int sy = p.px, sz = p.px * p.py;
     double M1[3] = {0.0, 0.0, 0.0}, sc[3] = {0.0, 0.0, 0.0};
     double M2[3][3] = {{0.0, 0.0, 0.0}, {0.0, 0.0, 0.0}, {0.0, 0.0, 0.0}};
     Unroll<0, L::Q>::run([&](auto nc) {

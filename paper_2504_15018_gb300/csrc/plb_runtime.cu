@@ -83,9 +83,13 @@ bool make_layout(int lattice, const int dims[3], int precision, Layout &L, int s
     off = align256(off + 4 * sizeof(double));
     L.off_staging = off;
     const int per_cell = L.Q > L.D + 2 ? L.Q : L.D + 2;
-    off = align256(off + (size_t)L.chunk * per_cell * sizeof(double));
+    // (a small lattice's staging area also serves as the second population copy of many-step launches)
+    const size_t staged = (size_t)L.chunk * per_cell * sizeof(double), copy = (size_t)L.Q * L.pstride * L.s_pop;
+    off = align256(off + (L.chunk == L.n && copy > staged ? copy : staged));
     L.off_flags = off;
     off = align256(off + 64);
+    L.off_counts = off;
+    off = align256(off + kTileWords * sizeof(unsigned));
     L.total = off;
     return true;
 }
@@ -127,6 +131,11 @@ template <class T> T *device_view(T *ptr) {
     if (a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged || a.type == cudaMemoryTypeHost)
         return static_cast<T *>(a.devicePointer);
     return nullptr;
+}
+
+// Counters of the many-step launch: all tiles at the same count (also after a wait that gave up).
+cudaError_t clear_counts(plb_t *h) {
+    return h->counts ? cudaMemsetAsync(h->counts, 0, plb::kTileWords * sizeof(unsigned), h->stream) : cudaSuccess;
 }
 
 int check_launch() {
@@ -400,8 +409,10 @@ int plb_create(int lattice, const int dims[3], const plb_eos_params *eos, double
     }
     h->opts.rho_ref = k.d.rho_ref;
     k.flags = reinterpret_cast<unsigned *>(h->ws + lay.off_flags);
+    h->counts = reinterpret_cast<unsigned *>(h->ws + lay.off_counts);
     cudaError_t e = cudaMemsetAsync(h->psi, 0, (size_t)lay.psi_elems * lay.s_psi, h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(k.flags, 0, 64, h->stream);
+    if (e == cudaSuccess) e = clear_counts(h);
     if (e == cudaSuccess && k.wall_fixed) {
         h->L->wall_fill(k, h->psi, h->stream);
         e = cudaGetLastError();
@@ -440,6 +451,7 @@ int plb::init_state(plb_state *h, const double *rho0, const double *u0) {
     // costs tens of milliseconds): flags cleared, first-invalid-index slots set to all ones
     PLB_CUDA(cudaMemsetAsync(h->kp.flags, 0, 64, h->stream));
     PLB_CUDA(cudaMemsetAsync(h->kp.flags + plb::FLAG_SLOT_RHO, 0xff, 16, h->stream));
+    PLB_CUDA(clear_counts(h));
     const double *drho0 = device_view(rho0), *du0 = u0 ? device_view(u0) : nullptr;
     if (drho0 && (!u0 || du0)) {
         // inputs the device can read: one launch over all cells
@@ -481,6 +493,56 @@ int plb::rebalance_state(plb_state *h) {
     return check_launch();
 }
 
+namespace {
+
+// Advances a small lattice by as many of n steps as the many-step launch takes (0: none).  In-place lattices borrow the staging area as the second population copy,
+// take an even number of steps (the populations end where they were) and start at even parity.
+int step_tiles(plb_t *h, int n, int coll) {
+    const int form = h->pops2 ? 1 : 0;
+    if (h->tiles_state == 0) {
+        const plb::Layout &L = h->lay;
+        bool use = h->counts && L.n == L.chunk;        // the staging area holds a second copy
+        if (use) use = h->L->tile_plan[form](h->kp, coll, h->tiles);
+        h->tiles_state = use ? 1 : -1;
+    }
+    if (h->tiles_state < 0) return 0;
+    plb::TileArgs t = h->tiles;
+    int first = 0;
+    if (!h->pops2) {
+        if (h->odd) {
+            // one in-place step brings the natural layout back
+            if (n < 3) return 0;
+            h->kp.salt = (unsigned)h->t;
+            h->L->psi(h->kp, h->pops, h->psi, 1, h->stream);
+            h->L->collide[coll](h->kp, h->pops, h->psi, 1, h->stream);
+            h->odd = 0;
+            h->t += 1;
+            first = 1;
+        }
+        t.nsteps = (n - first) & ~1;
+    } else {
+        t.nsteps = n;
+    }
+    if (t.nsteps < 2) return first;
+    t.a = h->pops;
+    t.b = h->pops2 ? h->pops2 : reinterpret_cast<char *>(h->staging);
+    t.counts = h->counts;
+    t.spin_limit = 1u << 22;
+    h->kp.salt = (unsigned)h->t;
+    cudaError_t e = h->L->tile_run[form](h->kp, coll, t, h->stream);
+    if (e != cudaSuccess) {
+        // the tiles do not fit this context (fewer SMs than the device reports): the other kernels do
+        cudaGetLastError();
+        h->tiles_state = -1;
+        return first;
+    }
+    if (h->pops2 && (t.nsteps & 1)) std::swap(h->pops, h->pops2);
+    h->t += t.nsteps;
+    return first + t.nsteps;
+}
+
+}  // namespace
+
 extern "C" {
 
 int plb_step(plb_t *h, int n) {
@@ -488,6 +550,7 @@ int plb_step(plb_t *h, int n) {
     if (h->view) return fail(PLB_EINVAL, "this lattice belongs to a batch: use plb_batch_step");
     if (h->slab) return fail(PLB_EINVAL, "this lattice is a slab: step it with plb_slab_pass and plb_slab_exchange");
     const int coll = h->opts.collision == PLB_MRT ? 1 : 0;
+    n -= step_tiles(h, n, coll);
     if (h->pops2) {
         // single pass: read the current copy, push into the other, swap
         for (int k = 0; k < n; ++k) {
@@ -556,6 +619,7 @@ int plb_status(plb_t *h) {
     unsigned flags = 0;
     PLB_CUDA(cudaMemcpyAsync(&flags, h->kp.flags, sizeof(unsigned), cudaMemcpyDeviceToHost, h->stream));
     PLB_CUDA(cudaStreamSynchronize(h->stream));
+    if (flags & plb::FLAG_TIMEOUT) return fail(PLB_ETIMEOUT, "a device-side wait of a step gave up");
     if (flags & plb::FLAG_NONFINITE) return fail(PLB_ENONFINITE, "a density became non-positive or non-finite");
     if (flags & plb::FLAG_PSI_DOMAIN) return fail(PLB_EPSI_DOMAIN, "2 (p_EOS - rho/3) / G < 0 on some cell");
     return PLB_OK;

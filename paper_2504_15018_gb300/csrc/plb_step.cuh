@@ -96,13 +96,12 @@ __device__ __forceinline__ void store_fast(const KParams &p, const Planes<S> &A,
     });
 }
 
-// Total force density from the padded psi field (pc points at the cell's psi).
+// Total force density from a psi field of row pitch sy and plane pitch sz (pc points at the cell's psi).
 template <class L, class T, class Pol = LdStream, class PsiT>
-__device__ __forceinline__ void force_fast(const KParams &p, const PsiT *__restrict__ pc, T F[3]) {
+__device__ __forceinline__ void force_fast(const KParams &p, const PsiT *__restrict__ pc, int sy, int sz, T F[3]) {
     const T psi0 = (T)Pol::ro(pc);
     T m1[3] = {0, 0, 0};
     T m2[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
-    const int sy = p.px, sz = p.px * p.py;
     Unroll<0, (L::Q - 1) / 2>::run([&](auto kc) {
         constexpr int i = 2 * decltype(kc)::value + 1;
         constexpr int cx = L::cx(i), cy = L::cy(i), cz = L::cz(i);
@@ -489,6 +488,21 @@ __device__ __forceinline__ void collide_emit(const KParams &p, T *f, const T F[3
 #define PLB_COLLIDE_MINB 3
 #endif
 
+// psi of a cell from its stored populations.
+template <class L, class S>
+__device__ __forceinline__ typename Store<S>::PsiT psi_cell(const KParams &p, const typename Store<S>::T *f) {
+    using T = typename Store<S>::T;
+    if constexpr (std::is_same<S, double>::value) {
+        return plain::psi(p, plain::density<L>(f));             // FP64: the plain evaluation
+    } else {
+        T rho = f[0];
+#pragma unroll
+        for (int i = 1; i < L::Q; ++i) rho += f[i];
+        if (Store<S>::SHIFT) rho += phys<T>(p).rho_ref;         // sum_i w_i rho_ref = rho_ref
+        return (typename Store<S>::PsiT)psi_of<T>(p, rho);
+    }
+}
+
 template <class L, class S, bool ODD, bool WALL, class Pol = LdStream, class I>
 __device__ __forceinline__ void psi_body(const KParams &p, const Planes<S> &A, typename Store<S>::PsiT *psi,
                                          const Geo<I> &g) {
@@ -496,16 +510,7 @@ __device__ __forceinline__ void psi_body(const KParams &p, const Planes<S> &A, t
     using PsiT = typename Store<S>::PsiT;
     T f[L::Q];
     load_fast<L, S, ODD, WALL, Pol>(p, A, g, f);
-    PsiT v;
-    if constexpr (std::is_same<S, double>::value) {
-        v = plain::psi(p, plain::density<L>(f));                // FP64: the plain evaluation
-    } else {
-        T rho = f[0];
-#pragma unroll
-        for (int i = 1; i < L::Q; ++i) rho += f[i];
-        if (Store<S>::SHIFT) rho += phys<T>(p).rho_ref;      // sum_i w_i rho_ref = rho_ref
-        v = (PsiT)psi_of<T>(p, rho);
-    }
+    const PsiT v = psi_cell<L, S>(p, f);
     psi[psi_index(p, g.x, g.y, g.z)] = v;
     // periodic images / wall mirrors in the ghost layer (boundary cells only)
     const bool bx = g.x == 0 || g.x == p.nx - 1, by = g.y == 0 || g.y == p.ny - 1;
@@ -556,10 +561,10 @@ __device__ __forceinline__ void collide_body(const KParams &p, const Planes<S> &
     T F[3];
     if constexpr (std::is_same<S, double>::value) {
         // FP64: the plain evaluation, term by term in the equations' order
-        plain::force<L, Pol>(p, psi + psi_index(p, g.x, g.y, g.z), F);
+        plain::force<L, Pol>(p, psi + psi_index(p, g.x, g.y, g.z), p.px, p.px * p.py, F);
         plain::collide<L, MRT>(p, f, F);
     } else {
-        force_fast<L, T, Pol>(p, psi + psi_index(p, g.x, g.y, g.z), F);
+        force_fast<L, T, Pol>(p, psi + psi_index(p, g.x, g.y, g.z), p.px, p.px * p.py, F);
         collide_fast<L, MRT, Store<S>::SHIFT, T>(p, f, F);
     }
     store_fast<L, S, ODD, WALL, SR>(p, A, g, f, salt);
