@@ -11,8 +11,10 @@ struct PrConstants {
 };
 
 PrConstants pr_constants(const plb_eos_params &e);
-double eos_pressure_host(const plb_eos_params &e, double rho);
 int solve_coexistence(const plb_eos_params &e, double &rho_v, double &rho_l, double &p0);
+// Whether a lattice with these options uses the coexistence densities: as the default FP16 shift, or
+// as the default densities of tau(rho).
+bool needs_coexistence(double tau, const plb_opts &o);
 int si_convert(const double si[6], const double lat[3], double xi, double out[11]);
 
 // Byte layout of the caller's device workspace (every region 256-byte aligned).

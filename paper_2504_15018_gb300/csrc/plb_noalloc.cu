@@ -75,8 +75,10 @@ extern "C" int plb_step_pairs_static(int lattice, const int dims[3], const plb_e
     st = scratch_address(&scratch);
     if (st != PLB_OK) return st;
 
+    // The solve takes milliseconds of host time on every call (this entry point keeps no handle):
+    // only where its densities are used.
     double rv = 0, rl = 0, p0 = 0;
-    if (plb::solve_coexistence(*eos, rv, rl, p0) != PLB_OK) rv = rl = 0;
+    if (plb::needs_coexistence(tau, o) && plb::solve_coexistence(*eos, rv, rl, p0) != PLB_OK) rv = rl = 0;
     plb::KParams k;
     st = plb::fill_kparams(dims, *eos, tau, G, eps, o, lay, rv, rl, k);
     if (st != PLB_OK) return st;

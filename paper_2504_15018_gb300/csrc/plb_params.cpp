@@ -27,18 +27,28 @@ PrConstants pr_constants(const plb_eos_params &e) {
     return c;
 }
 
-// p_EOS(rho) without p_scale.
-double eos_pressure_host(const plb_eos_params &e, double rho) {
-    if (e.kind == PLB_EOS_PR) {
-        const PrConstants c = pr_constants(e);
-        const double br = e.b * rho;
-        return rho * c.RT / (1.0 - br) - c.aalpha * rho * rho / (1.0 + 2.0 * br - br * br);
+// p_EOS(rho) without p_scale, with everything that does not depend on rho formed once: the solve
+// below evaluates it some 3e5 times, and forming the Peng-Robinson constants (a square root and
+// three divisions) in each took most of its 9 ms.
+namespace {
+struct Pressure {
+    const plb_eos_params &e;
+    const PrConstants c;
+    const double sv;
+    explicit Pressure(const plb_eos_params &eos)
+        : e(eos), c(eos.kind == PLB_EOS_PR ? pr_constants(eos) : PrConstants()), sv(std::sqrt(eos.rho_v)) {}
+    double operator()(double rho) const {
+        if (e.kind == PLB_EOS_PR) {
+            const double br = e.b * rho;
+            return rho * c.RT / (1.0 - br) - c.aalpha * rho * rho / (1.0 + 2.0 * br - br * br);
+        }
+        const double sr = std::sqrt(rho), rv = e.rho_v, rl = e.rho_l;
+        const double r2 = rho * rho;
+        return e.pc_over_rhoc3 * (2.0 * r2 * rho + (rv - 2.0 * rl) * r2 - 3.0 * sv * r2 * sr + 2.0 * sv * rl * rho * sr +
+                                  sv * rl * rl * sr);
     }
-    const double sr = std::sqrt(rho), sv = std::sqrt(e.rho_v), rv = e.rho_v, rl = e.rho_l;
-    const double r2 = rho * rho;
-    return e.pc_over_rhoc3 * (2.0 * r2 * rho + (rv - 2.0 * rl) * r2 - 3.0 * sv * r2 * sr + 2.0 * sv * rl * rho * sr +
-                              sv * rl * rl * sr);
-}
+};
+}  // namespace
 
 namespace {
 
@@ -46,9 +56,9 @@ double rho_upper(const plb_eos_params &e) {
     return e.kind == PLB_EOS_PR ? 0.999999 / e.b : 4.0 * e.rho_l;
 }
 
-double dpdrho(const plb_eos_params &e, double r) {
+double dpdrho(const Pressure &p, double r) {
     const double h = 1e-6 * r;
-    return (eos_pressure_host(e, r + h) - eos_pressure_host(e, r - h)) / (2.0 * h);
+    return (p(r + h) - p(r - h)) / (2.0 * h);
 }
 
 // root of g on [lo, hi] by bisection, g(lo) and g(hi) of opposite sign
@@ -68,19 +78,19 @@ template <class Fn> double bisect(Fn g, double lo, double hi, int iters = 200) {
     return 0.5 * (lo + hi);
 }
 
-bool spinodals(const plb_eos_params &e, double &s1, double &s2) {
-    const double top = rho_upper(e);
+bool spinodals(const Pressure &p, double &s1, double &s2) {
+    const double top = rho_upper(p.e);
     const int n = 4000;
-    double prev_r = top * 1e-6, prev_d = dpdrho(e, prev_r);
+    double prev_r = top * 1e-6, prev_d = dpdrho(p, prev_r);
     bool have1 = false;
     for (int k = 1; k <= n; ++k) {
         const double r = top * std::pow(10.0, -6.0 + 6.0 * k / n) * (1.0 - 1e-9);
-        const double d = dpdrho(e, r);
+        const double d = dpdrho(p, r);
         if (!have1 && prev_d > 0.0 && d <= 0.0) {
-            s1 = bisect([&](double x) { return dpdrho(e, x); }, prev_r, r);
+            s1 = bisect([&](double x) { return dpdrho(p, x); }, prev_r, r);
             have1 = true;
         } else if (have1 && prev_d < 0.0 && d >= 0.0) {
-            s2 = bisect([&](double x) { return dpdrho(e, x); }, prev_r, r);
+            s2 = bisect([&](double x) { return dpdrho(p, x); }, prev_r, r);
             return true;
         }
         prev_r = r;
@@ -112,18 +122,19 @@ int solve_coexistence(const plb_eos_params &e, double &rho_v, double &rho_l, dou
         return PLB_OK;
     }
     double s1 = 0, s2 = 0;
-    if (!spinodals(e, s1, s2)) return PLB_EINVAL;   // supercritical: no coexistence
+    const Pressure p(e);
+    if (!spinodals(p, s1, s2)) return PLB_EINVAL;   // supercritical: no coexistence
     const double top = rho_upper(e);
-    const double p_hi = eos_pressure_host(e, s1);
-    const double p_lo = std::fmax(eos_pressure_host(e, s2), 0.0);
+    const double p_hi = p(s1);
+    const double p_lo = std::fmax(p(s2), 0.0);
     auto roots = [&](double pp, double &rv, double &rl) {
-        rv = bisect([&](double r) { return eos_pressure_host(e, r) - pp; }, 0.0, s1);
-        rl = bisect([&](double r) { return eos_pressure_host(e, r) - pp; }, s2, top);
+        rv = bisect([&](double r) { return p(r) - pp; }, 0.0, s1);
+        rl = bisect([&](double r) { return p(r) - pp; }, s2, top);
     };
     auto area = [&](double pp) {
         double rv, rl;
         roots(pp, rv, rl);
-        auto g = [&](double r) { return (eos_pressure_host(e, r) - pp) / (r * r); };
+        auto g = [&](double r) { return (p(r) - pp) / (r * r); };
         // panels split at the spinodals; the vapour branch is graded geometrically
         double sum = 0.0;
         double a = rv;

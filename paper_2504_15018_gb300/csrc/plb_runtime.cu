@@ -252,6 +252,11 @@ int check_create_args(int lattice, const int dims[3], const plb_eos_params *eos,
     return PLB_OK;
 }
 
+bool needs_coexistence(double tau, const plb_opts &o) {
+    return (o.precision == PLB_FP16S && !(o.rho_ref > 0)) ||
+           (o.tau_v > 0.0 && o.tau_v != tau && !(o.tau_rho_l > o.tau_rho_v));
+}
+
 int fill_kparams(const int dims[3], const plb_eos_params &eos, double tau, double G, double eps, const plb_opts &o,
                  const Layout &lay, double rv, double rl, KParams &k) {
     std::memset(&k, 0, sizeof(k));
