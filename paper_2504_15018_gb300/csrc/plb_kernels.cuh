@@ -44,9 +44,17 @@
 
 namespace plb {
 
-// Linear thread -> cell mapping (x fastest) for the readout kernels.
+// Linear thread -> cell mapping (x fastest) for the readout kernels; 32-bit divisions where they do (the
+// 64-bit ones are about 100 instructions each).
 __device__ __forceinline__ bool cell_coords(const KParams &p, long long s, int &x, int &y, int &z) {
     if (s >= p.n) return false;
+    if (p.n < (1LL << 31)) {
+        const unsigned row = (unsigned)s / (unsigned)p.nx;
+        x = (int)((unsigned)s - row * (unsigned)p.nx);
+        z = (int)(row / (unsigned)p.ny);
+        y = (int)(row - (unsigned)z * (unsigned)p.ny);
+        return true;
+    }
     const long long plane = (long long)p.nx * p.ny;
     z = (int)(s / plane);
     const long long r = s - (long long)z * plane;
@@ -214,57 +222,92 @@ __global__ void k_set_pops(KParams p, S *__restrict__ A, const double *__restric
 }
 
 // ----------------------------------------------------------- reductions (a4)
-// Per-thread FP64 accumulation over a grid-stride loop, warp-shuffle tree, one
-// partial per block (4 doubles); plb_reduce_final sums the partials in block order.
-template <class L, class S>
-__global__ void __launch_bounds__(256) k_reduce(KParams p, const S *__restrict__ A,
-                                                const typename Store<S>::PsiT *__restrict__ psi, int odd, int what,
-                                                int lox, int loy, int loz, int hix, int hiy, int hiz,
-                                                double *__restrict__ partials) {
-    using T = typename Store<S>::T;
-    double acc[4] = {0, 0, 0, 0};
-    const bool is_max = (what == 2);
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x; s < p.n; s += stride) {
-        int x, y, z;
-        cell_coords(p, s, x, y, z);
-        if (x < lox || x >= hix || y < loy || y >= hiy || z < loz || z >= hiz) continue;
-        const Nbr nb = neighbours(p, x, y, z);
-        T f[L::Q];
-        load_pops<L, S>(p, A, x, y, z, nb, s, odd != 0, f);
-        double rho = 0, j[3] = {0, 0, 0};
-#pragma unroll
-        for (int i = 0; i < L::Q; ++i) rho += (double)f[i];
-        if (what >= 1 && what <= 4) {
-            // momentum only where it is used (GB300's FP64 rate is low); terms with a
-            // zero velocity component add exactly 0 and are skipped
-            Unroll<0, L::Q>::run([&](auto ic) {
-                constexpr int i = decltype(ic)::value;
-                if (L::cx(i) != 0) j[0] += (double)(L::cx(i) * f[i]);
-                if (L::cy(i) != 0) j[1] += (double)(L::cy(i) * f[i]);
-                if (L::cz(i) != 0) j[2] += (double)(L::cz(i) * f[i]);
-            });
-        }
-        if (what == 0 || what == 5) {
-            acc[0] += rho;
-        } else if (what == 6) {
-            acc[0] += (double)eos_pressure<T>(p, (T)rho);
-        } else {
-            T F[3];
-            cell_force<L, T>(p, psi, psi_index(p, x, y, z), F);
-            const double m[3] = {j[0] + 0.5 * (double)F[0], j[1] + 0.5 * (double)F[1], j[2] + 0.5 * (double)F[2]};
-            if (what == 1) {
-                acc[0] += m[0];
-                acc[1] += m[1];
-                acc[2] += m[2];
-            } else {
-                const double u2 = (m[0] * m[0] + m[1] * m[1] + m[2] * m[2]) / (rho * rho);
-                if (what == 2) acc[0] = fmax(acc[0], sqrt(u2));
-                else if (what == 3) acc[0] += sqrt(u2);
-                else acc[0] += u2;
-            }
-        }
+// A grid-stride loop per thread, warp-shuffle tree, one partial per block (4 doubles);
+// k_reduce_final sums the partials in block order.
+//
+// What bounds the sums is the FP64 pipe: two operations per clock and SM on GB300.  Adding every
+// population in FP64 took about 100 of them per cell, ten times the HBM time.  FP32 storage adds with
+// error-free transformations on the FP32 pipe instead and converts once per thread; the speed
+// maximum is searched in pairs of FP32 values, and FP64 evaluates the candidates only.  Mass, momentum,
+// maximum speed and moments of 256 x 128 x 128 cells, D3Q19 FP32: 2140 -> 800 us.
+
+// A sum of FP32 values in three FP32 parts, each the rounding error of the one before (TwoSum, Knuth
+// 1969; the cascade of Ogita, Rump and Oishi 2005): about 70 bits, where FP64 keeps 53.
+struct Sum3 {
+    float h = 0.0f, m = 0.0f, l = 0.0f;
+    __device__ __forceinline__ static float two_sum(float a, float b, float &err) {
+        const float s = __fadd_rn(a, b), bb = __fadd_rn(s, -a);
+        err = __fadd_rn(__fadd_rn(a, -__fadd_rn(s, -bb)), __fadd_rn(b, -bb));
+        return s;
     }
+    __device__ __forceinline__ void add(float x) {
+        float e1, e2;
+        h = two_sum(h, x, e1);
+        m = two_sum(m, e1, e2);
+        l = __fadd_rn(l, e2);
+    }
+    // (beyond FP32's range the error terms are NaN: the leading part then tells)
+    __device__ __forceinline__ double value() const {
+        return fabsf(h) < INFINITY ? (double)h + ((double)m + (double)l) : (double)h;
+    }
+    // the sum as a pair: hi the FP32 value nearest to it
+    __device__ __forceinline__ void pair(float &hi, float &lo) const {
+        hi = two_sum(h, __fadd_rn(m, l), lo);
+    }
+};
+
+// |momentum|^2 / rho^2 (scaled by 2^60) as a pair of FP32 values, relative error below 2^-40.
+__device__ __forceinline__ void speed2_pair(const Sum3 &rho, const Sum3 m[3], int dims, float &qh, float &ql) {
+    float nh = 0.0f, nl = 0.0f, e;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        if (a >= dims) continue;
+        float h, l;
+        m[a].pair(h, l);
+        h = __fmul_rn(h, 0x1p30f);
+        l = __fmul_rn(l, 0x1p30f);
+        const float s = __fmul_rn(h, h);
+        const float r = fmaf(h, h, -s) + 2.0f * h * l;
+        nh = Sum3::two_sum(nh, s, e);
+        nl += e + r;
+    }
+    nh = Sum3::two_sum(nh, nl, nl);
+    float rh, rl;
+    rho.pair(rh, rl);
+    const float dh = __fmul_rn(rh, rh), dl = fmaf(rh, rh, -dh) + 2.0f * rh * rl;
+    qh = __fdiv_rn(nh, dh);
+    ql = __fdiv_rn(fmaf(-qh, dl, fmaf(-qh, dh, nh) + nl), dh);
+    qh = Sum3::two_sum(qh, ql, ql);
+}
+
+// Density and total momentum (half the force included) of a cell in FP64.
+template <class L, class S>
+__device__ __forceinline__ void cell_sums(const KParams &p, const S *__restrict__ A,
+                                          const typename Store<S>::PsiT *__restrict__ psi, int odd, int what,
+                                          long long s, int x, int y, int z, double &rho, double m[3]) {
+    using T = typename Store<S>::T;
+    const Nbr nb = neighbours(p, x, y, z);
+    T f[L::Q];
+    load_pops<L, S>(p, A, x, y, z, nb, s, odd != 0, f);
+    rho = 0.0;
+    double j[3] = {0, 0, 0};
+#pragma unroll
+    for (int i = 0; i < L::Q; ++i) rho += (double)f[i];
+    if (what < 1 || what > 4) return;
+    // terms with a zero velocity component add exactly 0 and are skipped
+    Unroll<0, L::Q>::run([&](auto ic) {
+        constexpr int i = decltype(ic)::value;
+        if (L::cx(i) != 0) j[0] += (double)(L::cx(i) * f[i]);
+        if (L::cy(i) != 0) j[1] += (double)(L::cy(i) * f[i]);
+        if (L::cz(i) != 0) j[2] += (double)(L::cz(i) * f[i]);
+    });
+    T F[3];
+    cell_force<L, T>(p, psi, psi_index(p, x, y, z), F);
+    for (int a = 0; a < 3; ++a) m[a] = j[a] + 0.5 * (double)F[a];
+}
+
+// The block's partial from its threads' sums (or maxima).
+__device__ __forceinline__ void block_partial(double acc[4], bool is_max, double *__restrict__ partials) {
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
         double v = acc[c];
@@ -280,11 +323,117 @@ __global__ void __launch_bounds__(256) k_reduce(KParams p, const S *__restrict__
         for (int c = 0; c < 4; ++c) red[warp][c] = acc[c];
     __syncthreads();
     if (threadIdx.x < 4) {
-        double v = is_max ? 0.0 : 0.0;
+        double v = 0.0;
         const int nw = blockDim.x >> 5;
         for (int w = 0; w < nw; ++w) v = is_max ? fmax(v, red[w][threadIdx.x]) : v + red[w][threadIdx.x];
         partials[blockIdx.x * 4 + threadIdx.x] = v;
     }
+}
+
+struct Box {
+    int lo[3], hi[3];
+    __device__ __forceinline__ bool holds(int x, int y, int z) const {
+        return x >= lo[0] && x < hi[0] && y >= lo[1] && y < hi[1] && z >= lo[2] && z < hi[2];
+    }
+};
+
+// Every reduction, in FP64: FP64 storage, and the means of |u|, u^2 and the pressure.
+template <class L, class S>
+__global__ void __launch_bounds__(256) k_reduce(KParams p, const S *__restrict__ A,
+                                                const typename Store<S>::PsiT *__restrict__ psi, int odd, int what,
+                                                Box box, double *__restrict__ partials) {
+    using T = typename Store<S>::T;
+    double acc[4] = {0, 0, 0, 0};
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    for (long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x; s < p.n; s += stride) {
+        int x, y, z;
+        cell_coords(p, s, x, y, z);
+        if (!box.holds(x, y, z)) continue;
+        double rho, m[3];
+        cell_sums<L, S>(p, A, psi, odd, what, s, x, y, z, rho, m);
+        if (what == 0 || what == 5) {
+            acc[0] += rho;
+        } else if (what == 6) {
+            acc[0] += (double)eos_pressure<T>(p, (T)rho);
+        } else if (what == 1) {
+            acc[0] += m[0];
+            acc[1] += m[1];
+            acc[2] += m[2];
+        } else {
+            const double u2 = (m[0] * m[0] + m[1] * m[1] + m[2] * m[2]) / (rho * rho);
+            if (what == 2) acc[0] = fmax(acc[0], sqrt(u2));
+            else if (what == 3) acc[0] += sqrt(u2);
+            else acc[0] += u2;
+        }
+    }
+    block_partial(acc, what == 2, partials);
+}
+
+// FP32 arithmetic: density (WHAT 0), momentum (1) and the largest speed (2).
+template <class L, class S, int WHAT>
+__global__ void __launch_bounds__(256) k_reduce_f32(KParams p, const S *__restrict__ A, const float *__restrict__ psi,
+                                                    int odd, Box box, double *__restrict__ partials) {
+    double acc[4] = {0, 0, 0, 0};
+    Sum3 sum[3];
+    float bh = -1.0f, bl = 0.0f;               // WHAT 2: the largest speed^2 seen by this thread, its cell
+    long long best = -1;
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    for (long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x; s < p.n; s += stride) {
+        int x, y, z;
+        cell_coords(p, s, x, y, z);
+        if (!box.holds(x, y, z)) continue;
+        const Nbr nb = neighbours(p, x, y, z);
+        float f[L::Q];
+        load_pops<L, S>(p, A, x, y, z, nb, s, odd != 0, f);
+        if constexpr (WHAT == 0) {
+#pragma unroll
+            for (int i = 0; i < L::Q; ++i) sum[0].add(f[i]);
+        } else {
+            if (WHAT == 2) sum[0] = sum[1] = sum[2] = Sum3();
+            Unroll<0, L::Q>::run([&](auto ic) {
+                constexpr int i = decltype(ic)::value;
+                if (L::cx(i) != 0) sum[0].add(L::cx(i) * f[i]);
+                if (L::cy(i) != 0) sum[1].add(L::cy(i) * f[i]);
+                if (L::cz(i) != 0) sum[2].add(L::cz(i) * f[i]);
+            });
+            float F[3];
+            cell_force<L, float>(p, psi, psi_index(p, x, y, z), F);
+#pragma unroll
+            for (int a = 0; a < L::D; ++a) sum[a].add(0.5f * F[a]);
+            if constexpr (WHAT == 2) {
+                Sum3 rho;
+#pragma unroll
+                for (int i = 0; i < L::Q; ++i) rho.add(f[i]);
+                float qh, ql;
+                speed2_pair(rho, sum, L::D, qh, ql);
+                if (qh > bh || (qh == bh && ql > bl)) {
+                    bh = qh;
+                    bl = ql;
+                    best = s;
+                }
+            }
+        }
+    }
+    if constexpr (WHAT < 2) {
+#pragma unroll
+        for (int a = 0; a < (WHAT ? 3 : 1); ++a) acc[a] = sum[a].value();
+    } else {
+        // the threads whose cell comes within 2^-20 of the block's largest evaluate it in FP64
+        float top = bh;
+        for (int o = 16; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+        __shared__ float tops[8];
+        if ((threadIdx.x & 31) == 0) tops[threadIdx.x >> 5] = top;
+        __syncthreads();
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) top = fmaxf(top, tops[w]);
+        if (best >= 0 && bh >= top * (1.0f - 0x1p-20f)) {
+            int x, y, z;
+            double rho, m[3];
+            cell_coords(p, best, x, y, z);
+            cell_sums<L, S>(p, A, psi, odd, WHAT, best, x, y, z, rho, m);
+            acc[0] = fmax(0.0, sqrt((m[0] * m[0] + m[1] * m[1] + m[2] * m[2]) / (rho * rho)));
+        }
+    }
+    block_partial(acc, WHAT == 2, partials);
 }
 
 // Total mass of the whole lattice.  In either AA layout every population of every cell sits in
@@ -500,8 +649,24 @@ template <class L, class S> struct Launch {
     }
     static void reduce(const KParams &p, const void *A, const void *psi, int odd, int what, const int lo[3],
                        const int hi[3], double *partials, int nblocks, cudaStream_t st) {
-        k_reduce<L, S><<<nblocks, 256, 0, st>>>(p, (const S *)A, (const PsiT *)psi, odd, what, lo[0], lo[1], lo[2],
-                                                hi[0], hi[1], hi[2], partials);
+        const Box box = {{lo[0], lo[1], lo[2]}, {hi[0], hi[1], hi[2]}};
+        if constexpr (!std::is_same<S, double>::value) {
+            const S *a = (const S *)A;
+            const float *ps = (const float *)psi;
+            if (what == 0 || what == 5) {
+                k_reduce_f32<L, S, 0><<<nblocks, 256, 0, st>>>(p, a, ps, odd, box, partials);
+                return;
+            }
+            if (what == 1) {
+                k_reduce_f32<L, S, 1><<<nblocks, 256, 0, st>>>(p, a, ps, odd, box, partials);
+                return;
+            }
+            if (what == 2) {
+                k_reduce_f32<L, S, 2><<<nblocks, 256, 0, st>>>(p, a, ps, odd, box, partials);
+                return;
+            }
+        }
+        k_reduce<L, S><<<nblocks, 256, 0, st>>>(p, (const S *)A, (const PsiT *)psi, odd, what, box, partials);
     }
     static void mass(const KParams &p, const void *A, double *partials, int nblocks, cudaStream_t st) {
         k_mass_flat<L, S><<<nblocks, 256, 0, st>>>(p, (const S *)A, partials);

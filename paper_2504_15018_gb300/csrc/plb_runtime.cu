@@ -80,7 +80,7 @@ bool make_layout(int lattice, const int dims[3], int precision, Layout &L, int s
     L.off_partials = off;
     off = align256(off + (size_t)L.max_blocks * 4 * sizeof(double));
     L.off_out = off;
-    off = align256(off + 4 * sizeof(double));
+    off = align256(off + 5 * sizeof(double));
     L.off_staging = off;
     const int per_cell = L.Q > L.D + 2 ? L.Q : L.D + 2;
     // (a small lattice's staging area also serves as the second population copy of many-step launches)
@@ -98,7 +98,8 @@ bool make_layout(int lattice, const int dims[3], int precision, Layout &L, int s
 
 namespace {
 
-void reduce_final_launch(const double *partials, int nblocks, int is_max, double *out, cudaStream_t st);
+void reduce_final_launch(const double *partials, int nblocks, int is_max, const unsigned *flags, double *out,
+                         cudaStream_t st);
 
 const plb::Launchers *launchers_for(int lattice, int precision) {
     switch (precision) {
@@ -619,15 +620,19 @@ int plb_step_timed(plb_t *h, int n, double ms[2]) {
     return st;
 }
 
+static int status_of(unsigned flags) {
+    if (flags & plb::FLAG_TIMEOUT) return fail(PLB_ETIMEOUT, "a device-side wait of a step gave up");
+    if (flags & plb::FLAG_NONFINITE) return fail(PLB_ENONFINITE, "a density became non-positive or non-finite");
+    if (flags & plb::FLAG_PSI_DOMAIN) return fail(PLB_EPSI_DOMAIN, "2 (p_EOS - rho/3) / G < 0 on some cell");
+    return PLB_OK;
+}
+
 int plb_status(plb_t *h) {
     if (!h) return fail(PLB_EINVAL, "NULL handle");
     unsigned flags = 0;
     PLB_CUDA(cudaMemcpyAsync(&flags, h->kp.flags, sizeof(unsigned), cudaMemcpyDeviceToHost, h->stream));
     PLB_CUDA(cudaStreamSynchronize(h->stream));
-    if (flags & plb::FLAG_TIMEOUT) return fail(PLB_ETIMEOUT, "a device-side wait of a step gave up");
-    if (flags & plb::FLAG_NONFINITE) return fail(PLB_ENONFINITE, "a density became non-positive or non-finite");
-    if (flags & plb::FLAG_PSI_DOMAIN) return fail(PLB_EPSI_DOMAIN, "2 (p_EOS - rho/3) / G < 0 on some cell");
-    return PLB_OK;
+    return status_of(flags);
 }
 
 int plb_moments(plb_t *h, double *rho, double *u, double *p) {
@@ -643,7 +648,6 @@ int plb_moments(plb_t *h, double *rho, double *u, double *p) {
         h->L->moments(h->kp, pops_ptr(h), psi_ptr(h), h->odd, drho, du, dp, 0, n, h->stream);
         int st = check_launch();
         if (st) return st;
-        PLB_CUDA(cudaStreamSynchronize(h->stream));
         return plb_status(h);
     }
     double *stg = staging_ptr(h);
@@ -690,10 +694,10 @@ int plb_reduce(plb_t *h, int what, const int lo[3], const int hi[3], double *out
         h->L->reduce(h->kp, pops_ptr(h), psi_ptr(h), h->odd, what, blo, bhi, partials, nblocks, h->stream);
     int st = check_launch();
     if (st) return st;
-    reduce_final_launch(partials, nblocks, what == PLB_UMAX, dout, h->stream);
+    reduce_final_launch(partials, nblocks, what == PLB_UMAX, h->kp.flags, dout, h->stream);
     st = check_launch();
     if (st) return st;
-    double res[4];
+    double res[5];                 // four sums or maxima, the error flags
     PLB_CUDA(cudaMemcpyAsync(res, dout, sizeof(res), cudaMemcpyDeviceToHost, h->stream));
     PLB_CUDA(cudaStreamSynchronize(h->stream));
     switch (what) {
@@ -703,7 +707,7 @@ int plb_reduce(plb_t *h, int what, const int lo[3], const int hi[3], double *out
         case PLB_MEAN_P: out[0] = res[0] / (double)count; break;
         default: out[0] = res[0];
     }
-    return plb_status(h);
+    return status_of((unsigned)res[4]);
 }
 
 int plb_get_populations(plb_t *h, double *f) {
@@ -778,17 +782,25 @@ int plb_set_state(plb_t *h, const void *host_buf, size_t bytes) {
 
 }  // extern "C"
 
-// Final pass of the reductions: one warp sums the block partials in a fixed order.
+// Final pass of the reductions: one warp per component sums every 32nd block's partial in each lane,
+// then the lanes, in a fixed order (one thread adding all 1024 in turn is a 30 us chain of FP64
+// additions).  The lattice's error flags ride along in out[4].
 namespace {
-__global__ void k_reduce_final(const double *__restrict__ partials, int nblocks, int is_max, double *__restrict__ out) {
-    const int c = threadIdx.x;
-    if (c >= 4) return;
+__global__ void k_reduce_final(const double *__restrict__ partials, int nblocks, int is_max,
+                               const unsigned *__restrict__ flags, double *__restrict__ out) {
+    const int c = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double v = 0.0;
-    for (int b = 0; b < nblocks; ++b) v = is_max ? fmax(v, partials[b * 4 + c]) : v + partials[b * 4 + c];
-    out[c] = v;
+    for (int b = lane; b < nblocks; b += 32) v = is_max ? fmax(v, partials[b * 4 + c]) : v + partials[b * 4 + c];
+    for (int o = 16; o > 0; o >>= 1) {
+        const double w = __shfl_down_sync(0xffffffffu, v, o);
+        v = is_max ? fmax(v, w) : v + w;
+    }
+    if (lane == 0) out[c] = v;
+    if (threadIdx.x == 0) out[4] = (double)*flags;
 }
 
-void reduce_final_launch(const double *partials, int nblocks, int is_max, double *out, cudaStream_t st) {
-    k_reduce_final<<<1, 32, 0, st>>>(partials, nblocks, is_max, out);
+void reduce_final_launch(const double *partials, int nblocks, int is_max, const unsigned *flags, double *out,
+                         cudaStream_t st) {
+    k_reduce_final<<<1, 128, 0, st>>>(partials, nblocks, is_max, flags, out);
 }
 }  // namespace
