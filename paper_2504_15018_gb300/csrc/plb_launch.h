@@ -26,6 +26,11 @@ template <class T> struct Phys {
     T psi_wall;               // psi on wetting walls (used when KParams::wall_fixed)
 };
 
+// 1 / b of a divisor b: the double nearest to it and the rest.
+struct Recip {
+    double h, l;
+};
+
 // Constants of the plain FP64 evaluation (plb_plain.cuh), each formed on the host the way
 // the equations write it.
 struct PlainPhys {
@@ -35,7 +40,8 @@ struct PlainPhys {
     double p_scale, G;
     double K1, K2;                             // G/12 (2 kappa - 2 - 3 eps), G/6 (kappa - 1)
     double tau_l, tau_v, tau_rho_v, d_rho, d_tau;   // tau(rho): rho_l - rho_v, tau_l - tau_v
-    double s_rate[6];                          // MRT rates by kind (1..5)
+    double s_rate[6], s_half[6];               // MRT rates s by kind (1..5), 1 - s / 2
+    Recip inv_G, inv_tau, inv_d_rho;           // of G, tau_l and d_rho
     double fext[3];
 };
 

@@ -17,6 +17,18 @@
 //    conserved rows relaxed with 1/tau like the stress rows).
 // Zero terms (a zero velocity component or basis coefficient) are skipped: adding an exact
 // zero to a sum that starts at +0 changes no bit.
+//
+// What bounds these kernels is the FP64 pipe (2 operations per clock and SM), so every operation that
+// cannot change a bit is left out:
+//  - a sum starts with its first term, not with 0 + term;
+//  - a product that differs in sign only from one at hand (opposite velocities, signs of the basis and
+//    of c) is that one, subtracted;
+//  - a product with a power of two is exact, so product and sum are one fused multiply-add;
+//  - a division by a number used often (tau, G, 3, the density span of tau(rho)) multiplies by its
+//    reciprocal, held as a pair of doubles, and corrects the quotient by its exact remainder: four
+//    operations for the correctly rounded quotient (Markstein 1990; quotient below).
+// Microseconds a step: 96^3 D3Q19 MRT 2640 -> 2300, 301 x 203 D2Q9 BGK with tau(rho) 69 -> 59; the same
+// bits.
 #pragma once
 #include "plb_device.cuh"
 
@@ -98,6 +110,13 @@ template <class L> __host__ __device__ constexpr double basis_norm2(int k) {
     return s;
 }
 
+// Whether velocity n is the first with a non-zero entry in row k.
+template <class L> __host__ __device__ constexpr bool first_entry(int k, int n) {
+    for (int m = 0; m < n; ++m)
+        if (basis<L>(k, m) != 0.0) return false;
+    return true;
+}
+
 // Relaxation rate of row k: 0 = 1/tau (conserved and stress rows), else the Phys::s_rate kind.
 template <class L> __host__ __device__ constexpr int rate_kind(int k) {
     if (L::Q == 9) return k == 1 ? 1 : k == 2 ? 2 : (k == 4 || k == 6) ? 3 : 0;
@@ -124,10 +143,32 @@ __host__ __device__ inline double psi_arg(const PlainPhys &q, int eos_kind, doub
     return 2.0 * (pressure(q, eos_kind, rho) - rho / 3.0) / q.G;
 }
 
+// a / b, rounded to nearest.  rh + rl is 1 / b (rh the double nearest to it, rl the rest), so
+// q = RN(a rh + RN(a rl)) misses a / b by less than half an ulp and 2^-50 ulp: it is one of the two doubles
+// around a / b, its remainder a - q b is a double, and RN(q + remainder rh) is the nearest one
+// (Markstein 1990, theorem on the final step).  For a outside 2^-900 .. 2^900 or b outside 2^-100 ..
+// 2^100, where a remainder could be subnormal or a product overflow, the division itself.  (The tests
+// are on the exponents, off the FP64 pipe.)
+__device__ __forceinline__ double quotient(double a, double b, const Recip &r) {
+    const unsigned hi = (unsigned)__double2hiint(a), er = ((unsigned)__double2hiint(r.h) >> 20) & 0x7ffu;
+    const bool zero = (hi << 1 | (unsigned)__double2loint(a)) == 0u;
+    if (((hi >> 20 & 0x7ffu) - 123u >= 1800u && !zero) || er - 923u >= 200u) return a / b;
+    const double q = __fma_rn(a, r.h, __dmul_rn(a, r.l));
+    return __fma_rn(__fma_rn(-b, q, a), r.h, q);
+}
+
+// 1 / b as a pair of doubles.
+__host__ __device__ inline Recip reciprocal(double b) {
+    Recip r;
+    r.h = 1.0 / b;
+    r.l = fma(-b, r.h, 1.0) * r.h;
+    return r;
+}
+
 // rho of Eq. Density.
 template <class L> __device__ __forceinline__ double density(const double *f) {
-    double r = 0.0;
-    Unroll<0, L::Q>::run([&](auto nc) { r = r + f[Order<L>::slot(decltype(nc)::value)]; });
+    double r = f[Order<L>::slot(0)];
+    Unroll<1, L::Q>::run([&](auto nc) { r = r + f[Order<L>::slot(decltype(nc)::value)]; });
     return r;
 }
 
@@ -137,12 +178,28 @@ __device__ __forceinline__ double psi(const KParams &p, double rho) {
         atomicOr(p.flags, FLAG_NONFINITE);
         return 0.0;
     }
-    const double arg = psi_arg(p.pl, p.eos_kind, rho);
+    // psi_arg, its divisions by 3 and by G through their reciprocals
+    constexpr double third = 1.0 / 3.0;
+    const Recip r3 = {third, 0x1.5555555555555p-56};
+    const double arg = quotient(2.0 * (pressure(p.pl, p.eos_kind, rho) - quotient(rho, 3.0, r3)), p.pl.G, p.pl.inv_G);
     if (!(arg >= 0.0)) {
         atomicOr(p.flags, FLAG_PSI_DOMAIN);
         return 0.0;
     }
     return sqrt(arg);
+}
+
+// Whether velocity n is the first of the summation order with a non-zero c_a (c_a c_b).
+template <class L> __host__ __device__ constexpr bool first_of(int n, int a, int b) {
+    for (int m = 0; m < n; ++m)
+        if (cc<L>(m, a) * cc<L>(m, b) != 0) return false;
+    return true;
+}
+
+// sum = sum +- term; the first term of a sum starts it.
+template <bool FIRST, bool PLUS> __device__ __forceinline__ void add_term(double &sum, double term) {
+    if (FIRST) sum = PLUS ? term : -term;
+    else sum = PLUS ? sum + term : sum - term;
 }
 
 // Total force density at a cell (Eqs. Shan_Chen_Force, interactionForce, plus the body
@@ -151,30 +208,30 @@ template <class L, class Pol>
 __device__ __forceinline__ void force(const KParams &p, const double *__restrict__ pc, int sy, int sz, double F[3]) {
     constexpr int D = L::D;
     const PlainPhys &q = p.pl;
-    double M1[3] = {0.0, 0.0, 0.0}, sc[3] = {0.0, 0.0, 0.0};
-    double M2[3][3] = {{0.0, 0.0, 0.0}, {0.0, 0.0, 0.0}, {0.0, 0.0, 0.0}};
+    double M1[3], sc[3], M2[3][3];
     Unroll<0, L::Q>::run([&](auto nc) {
         constexpr int n = decltype(nc)::value;
-        constexpr int c[3] = {cc<L>(n, 0), cc<L>(n, 1), cc<L>(n, 2)};
-        const double pn = Pol::ro(pc + (c[0] + c[1] * sy + c[2] * sz));
+        const double pn = Pol::ro(pc + (cc<L>(n, 0) + cc<L>(n, 1) * sy + cc<L>(n, 2) * sz));
         const double wp = L::w(Order<L>::slot(n)) * pn;
-#pragma unroll
-        for (int a = 0; a < D; ++a) {
-            if (c[a] != 0) M1[a] = M1[a] + wp * (double)c[a] * 3.0;
-#pragma unroll
-            for (int b = a; b < D; ++b)
-                if (cc2<L>(n, a, b) != 0.0) M2[a][b] = M2[a][b] + wp * cc2<L>(n, a, b) * 9.0;
-        }
-        if (n > 0) {
-#pragma unroll
-            for (int a = 0; a < D; ++a)
-                if (c[a] != 0) sc[a] = sc[a] + omega_sc<L>(n) * pn * (double)c[a];
-        }
+        const double w3 = wp * 3.0, w9 = wp * 9.0, os = omega_sc<L>(n) * pn;
+        const double full = wp * (1.0 - CS2) * 9.0, part = wp * (0.0 - CS2) * 9.0;   // a = b, c_a != 0 or = 0
+        Unroll<0, D>::run([&](auto ac) {
+            constexpr int a = decltype(ac)::value, ca = cc<L>(n, a);
+            if constexpr (ca != 0) {
+                add_term<first_of<L>(n, a, a), (ca > 0)>(M1[a], w3);
+                add_term<first_of<L>(n, a, a), (ca > 0)>(sc[a], os);
+            }
+            add_term<n == 0, true>(M2[a][a], ca != 0 ? full : part);
+            Unroll<a + 1, D>::run([&](auto bc) {
+                constexpr int b = decltype(bc)::value, cab = ca * cc<L>(n, b);
+                if constexpr (cab != 0) add_term<first_of<L>(n, a, b), (cab > 0)>(M2[a][b], w9);
+            });
+        });
     });
     const double psi0 = Pol::ro(pc);
-    double trM2 = 0.0;
+    double trM2 = M2[0][0];
 #pragma unroll
-    for (int b = 0; b < D; ++b) trM2 = trM2 + M2[b][b];
+    for (int b = 1; b < D; ++b) trM2 = trM2 + M2[b][b];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         if (a >= D) {
@@ -182,46 +239,93 @@ __device__ __forceinline__ void force(const KParams &p, const double *__restrict
             continue;
         }
         const double Fsc = -q.G * psi0 * sc[a];
-        double M1M2 = 0.0;
+        double M1M2 = M1[0] * M2[0][a];
 #pragma unroll
-        for (int b = 0; b < D; ++b) M1M2 = M1M2 + M1[b] * (a <= b ? M2[a][b] : M2[b][a]);
+        for (int b = 1; b < D; ++b) M1M2 = M1M2 + M1[b] * (a <= b ? M2[a][b] : M2[b][a]);
         const double Fint = Fsc - q.K1 * M1M2 + q.K2 * M1[a] * trM2;
         F[a] = Fint + q.fext[a];
     }
 }
 
-// f^eq_n of Eq. Single_Phase_EDF, n in the summation order.
-template <class L, int n> __device__ __forceinline__ double feq(double rho, const double u[3]) {
-    constexpr int D = L::D;
-    double cu = 0.0, quad = 0.0;
-#pragma unroll
-    for (int a = 0; a < D; ++a) {
-        if (cc<L>(n, a) > 0) cu = cu + u[a];
-        if (cc<L>(n, a) < 0) cu = cu - u[a];
-    }
-#pragma unroll
-    for (int a = 0; a < D; ++a)
-#pragma unroll
-        for (int b = 0; b < D; ++b)
-            if (cc2<L>(n, a, b) != 0.0) quad = quad + cc2<L>(n, a, b) * u[a] * u[b];
-    return L::w(Order<L>::slot(n)) * rho * (1.0 + cu * 3.0 + quad * 4.5);
+// Component a of the velocity of storage slot i.
+template <class L> __host__ __device__ constexpr int cs(int i, int a) {
+    return a == 0 ? L::cx(i) : (a == 1 ? L::cy(i) : L::cz(i));
 }
 
-// The bracket of Eq. Guo_Forcing_Scheme (without 1 - 1/(2 tau)), n in the summation order.
-template <class L, int n> __device__ __forceinline__ double guo(const double F[3], const double u[3]) {
-    constexpr int D = L::D;
-    double cF = 0.0, quad = 0.0;
+// The products (c_a c_b - c_s^2 d_ab) x_a y_b that the quadratic terms sum: a = b with c_a != 0 (full)
+// and c_a = 0 (part), and a != b up to sign (off).
+template <class L> struct Products {
+    double full[3], part[3], off[3][3];
+    __device__ __forceinline__ Products(const double *x, const double *y) {
 #pragma unroll
-    for (int a = 0; a < D; ++a) {
-        if (cc<L>(n, a) > 0) cF = cF + F[a];
-        if (cc<L>(n, a) < 0) cF = cF - F[a];
+        for (int a = 0; a < L::D; ++a) {
+            full[a] = (1.0 - CS2) * x[a] * y[a];
+            part[a] = (0.0 - CS2) * x[a] * y[a];
+#pragma unroll
+            for (int b = 0; b < L::D; ++b)
+                if (a != b) off[a][b] = x[a] * y[b];
+        }
     }
-#pragma unroll
-    for (int a = 0; a < D; ++a)
-#pragma unroll
-        for (int b = 0; b < D; ++b)
-            if (cc2<L>(n, a, b) != 0.0) quad = quad + cc2<L>(n, a, b) * F[a] * u[b];
-    return L::w(Order<L>::slot(n)) * (cF * 3.0 + quad * 9.0);
+    // their sum for the velocity of storage slot I (the same for -c)
+    template <int I> __device__ __forceinline__ double sum() const {
+        double s;
+        Unroll<0, L::D>::run([&](auto ac) {
+            constexpr int a = decltype(ac)::value;
+            Unroll<0, L::D>::run([&](auto bc) {
+                constexpr int b = decltype(bc)::value, cab = cs<L>(I, a) * cs<L>(I, b);
+                if constexpr (a == b) add_term<a == 0, true>(s, cab != 0 ? full[a] : part[a]);
+                else if constexpr (cab != 0) add_term<false, (cab > 0)>(s, off[a][b]);
+            });
+        });
+        return s;
+    }
+};
+
+// c . x for the velocity of storage slot I.
+template <class L, int I> __device__ __forceinline__ double along(const double *x) {
+    double s = 0.0;
+    Unroll<0, L::D>::run([&](auto ac) {
+        constexpr int a = decltype(ac)::value;
+        constexpr bool one = (a == 0 || cs<L>(I, 0) == 0) && (a <= 1 || cs<L>(I, 1) == 0);
+        if constexpr (cs<L>(I, a) != 0) add_term<one, (cs<L>(I, a) > 0)>(s, x[a]);
+    });
+    return s;
+}
+
+// f^eq of Eq. Single_Phase_EDF into storage slots; opposite velocities (slots i, i + 1) share their terms.
+template <class L> __device__ __forceinline__ void equilibrium(double rho, const double u[3], double *fe) {
+    const Products<L> uu(u, u);
+    fe[0] = L::w(0) * rho * (1.0 + uu.template sum<0>() * 4.5);
+    Unroll<0, (L::Q - 1) / 2>::run([&](auto rc) {
+        constexpr int i = 2 * decltype(rc)::value + 1;
+        const double cu = along<L, i>(u) * 3.0, quad = uu.template sum<i>() * 4.5, wr = L::w(i) * rho;
+        fe[i] = wr * (1.0 + cu + quad);
+        fe[i + 1] = wr * (1.0 - cu + quad);
+    });
+}
+
+// The bracket of Eq. Guo_Forcing_Scheme (without 1 - 1/(2 tau)) into storage slots.
+template <class L> __device__ __forceinline__ void guo(const double F[3], const double u[3], double *Ft) {
+    const Products<L> Fu(F, u);
+    Ft[0] = L::w(0) * (Fu.template sum<0>() * 9.0);
+    Unroll<0, (L::Q - 1) / 2>::run([&](auto rc) {
+        constexpr int i = 2 * decltype(rc)::value + 1;
+        const double cF = along<L, i>(F) * 3.0, quad = Fu.template sum<i>() * 9.0;
+        Ft[i] = L::w(i) * (cF + quad);
+        Ft[i + 1] = L::w(i) * (quad - cF);
+    });
+}
+
+// Whether |v| is a power of two (basis entries: 1, 2, 4, 8 among others).
+__host__ __device__ constexpr bool is_pow2(double v) {
+    v = v < 0 ? -v : v;
+    return v == 1.0 || v == 2.0 || v == 4.0 || v == 8.0;
+}
+
+// sum + m x for a basis entry m, rounded after the product and after the sum.
+template <bool FIRST> __device__ __forceinline__ double project(double m, double x, double sum) {
+    if (FIRST) return m * x;
+    return is_pow2(m) ? __fma_rn(m, x, sum) : sum + m * x;
 }
 
 // In place: pre-collision populations f (storage slots) -> post-collision populations.
@@ -230,75 +334,65 @@ template <class L, int MRT> __device__ __forceinline__ void collide(const KParam
     const PlainPhys &q = p.pl;
     const double rho = density<L>(f);
     double u[3] = {0.0, 0.0, 0.0};
-#pragma unroll
-    for (int a = 0; a < D; ++a) {
-        double m = 0.0;
+    Unroll<0, D>::run([&](auto ac) {
+        constexpr int a = decltype(ac)::value;
+        double m;
         Unroll<0, Q>::run([&](auto nc) {
             constexpr int n = decltype(nc)::value;
-            if (cc<L>(n, a) > 0) m = m + f[Order<L>::slot(n)];
-            if (cc<L>(n, a) < 0) m = m - f[Order<L>::slot(n)];
+            if constexpr (cc<L>(n, a) != 0) add_term<first_of<L>(n, a, a), (cc<L>(n, a) > 0)>(m, f[Order<L>::slot(n)]);
         });
         u[a] = (m + F[a] / 2.0) / rho;
-    }
+    });
     double tau = q.tau_l;
+    Recip itau = q.inv_tau;
     if (p.var_tau) {
-        double wgt = (rho - q.tau_rho_v) / q.d_rho;
+        double wgt = quotient(rho - q.tau_rho_v, q.d_rho, q.inv_d_rho);
         if (wgt < 0.0) wgt = 0.0;
         if (wgt > 1.0) wgt = 1.0;
         tau = q.tau_v + wgt * q.d_tau;
+        itau = reciprocal(tau);
     }
+    double fneq[Q], Ft[Q];
+    equilibrium<L>(rho, u, fneq);
+    guo<L>(F, u, Ft);
+#pragma unroll
+    for (int i = 0; i < Q; ++i) fneq[i] = f[i] - fneq[i];
     if constexpr (!MRT) {
-        const double kg = 1.0 - 1.0 / (2.0 * tau);
-        Unroll<0, Q>::run([&](auto nc) {
-            constexpr int n = decltype(nc)::value;
-            constexpr int i = Order<L>::slot(n);
-            const double fe = feq<L, n>(rho, u);
-            const double Fi = kg * guo<L, n>(F, u);
-            f[i] = f[i] - (f[i] - fe) / tau + Fi;
-        });
+        const double kg = 1.0 - 0.5 * itau.h;                    // 1 / (2 tau) is half of 1 / tau
+#pragma unroll
+        for (int i = 0; i < Q; ++i) f[i] = f[i] - quotient(fneq[i], tau, itau) + kg * Ft[i];
     } else {
-        double fneq[Q], Ft[Q], dmf[Q];
-        Unroll<0, Q>::run([&](auto nc) {
-            constexpr int n = decltype(nc)::value;
-            fneq[n] = f[Order<L>::slot(n)] - feq<L, n>(rho, u);
-            Ft[n] = guo<L, n>(F, u);
-        });
-        const double s_tau = 1.0 / tau;
+        // row by row: moments of f - f^eq and of the bracket, and their part of M^-1
+        double corr[Q];
         Unroll<0, Q>::run([&](auto kc) {
             constexpr int k = decltype(kc)::value;
             double mneq = 0.0, mf = 0.0;
             Unroll<0, Q>::run([&](auto nc) {
                 constexpr int n = decltype(nc)::value;
                 constexpr double m = basis<L>(k, n);
-                if (m != 0.0) {
-                    mneq = mneq + m * fneq[n];
-                    mf = mf + m * Ft[n];
+                if constexpr (m != 0.0) {
+                    constexpr bool one = first_entry<L>(k, n);
+                    mneq = project<one>(m, fneq[Order<L>::slot(n)], mneq);
+                    mf = project<one>(m, Ft[Order<L>::slot(n)], mf);
                 }
             });
-            const double s = rate_kind<L>(k) == 0 ? s_tau : q.s_rate[rate_kind<L>(k)];
+            constexpr int kind = rate_kind<L>(k);
+            const double s = kind == 0 ? itau.h : q.s_rate[kind];
+            const double half = kind == 0 ? 1.0 - itau.h / 2.0 : q.s_half[kind];
             const double dm = s * mneq;
-            const double mF = (1.0 - s / 2.0) * mf;
-            dmf[k] = mF - dm;
+            const double mF = half * mf;
+            const double dmf = mF - dm;
+            Unroll<0, Q>::run([&](auto nc) {
+                constexpr int n = decltype(nc)::value;
+                constexpr double mi = basis<L>(k, n) / basis_norm2<L>(k);
+                if constexpr (mi != 0.0) add_term<k == 0, (mi > 0.0)>(corr[n], (mi > 0.0 ? mi : -mi) * dmf);
+            });
         });
         Unroll<0, Q>::run([&](auto nc) {
             constexpr int n = decltype(nc)::value;
-            double corr = 0.0;
-            Unroll<0, Q>::run([&](auto kc) {
-                constexpr int k = decltype(kc)::value;
-                constexpr double mi = basis<L>(k, n) / basis_norm2<L>(k);
-                if (mi != 0.0) corr = corr + mi * dmf[k];
-            });
-            f[Order<L>::slot(n)] = f[Order<L>::slot(n)] + corr;
+            f[Order<L>::slot(n)] = f[Order<L>::slot(n)] + corr[n];
         });
     }
-}
-
-// f = f^eq(rho, u) of Eq. Single_Phase_EDF into storage slots (initialisation).
-template <class L> __device__ __forceinline__ void equilibrium(double rho, const double u[3], double *f) {
-    Unroll<0, L::Q>::run([&](auto nc) {
-        constexpr int n = decltype(nc)::value;
-        f[Order<L>::slot(n)] = feq<L, n>(rho, u);
-    });
 }
 
 }  // namespace plain

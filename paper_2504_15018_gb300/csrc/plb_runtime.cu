@@ -341,7 +341,13 @@ int fill_kparams(const int dims[3], const plb_eos_params &eos, double tau, doubl
     pl.tau_rho_v = trv;
     pl.d_rho = trl - trv;
     pl.d_tau = tau - d.tau_v;
-    for (int r = 0; r < 6; ++r) pl.s_rate[r] = d.s_rate[r];
+    for (int r = 0; r < 6; ++r) {
+        pl.s_rate[r] = d.s_rate[r];
+        pl.s_half[r] = 1.0 - d.s_rate[r] / 2.0;
+    }
+    pl.inv_G = plain::reciprocal(G);
+    pl.inv_tau = plain::reciprocal(tau);
+    pl.inv_d_rho = k.var_tau ? plain::reciprocal(pl.d_rho) : Recip{0.0, 0.0};
     for (int a = 0; a < 3; ++a) pl.fext[a] = d.fext[a];
     if (k.wall_fixed) {
         // Eq. Interaction_Potential at the wall density
