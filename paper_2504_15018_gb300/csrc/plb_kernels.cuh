@@ -533,12 +533,8 @@ template <class L, class S> struct Launch {
         dim3 grid, block;
         if constexpr (std::is_same<S, __half>::value) {
             if (PLB_PSI_QUAD && p.nx % 4 == 0 && p.n < (1LL << 31)) {
-                const int nq = p.nx / 4;
-                const int bx = nq >= 64 ? 64 : (nq + 31) / 32 * 32;
-                int by = 256 / bx;
-                if (by > p.ny) by = p.ny;
-                k_psi_quad<L, ODD><<<dim3((nq + bx - 1) / bx, (p.ny + by - 1) / by, p.nzl), dim3(bx, by), 0, st>>>(
-                    p, planes(p, A), (float *)psi);
+                const long long quads = (long long)(p.nx / 4) * p.ny;
+                k_psi_quad<L, ODD><<<dim3(blocks(quads, 256), 1, p.nzl), 256, 0, st>>>(p, planes(p, A), (float *)psi);
                 return;
             }
         }
@@ -571,22 +567,28 @@ template <class L, class S> struct Launch {
         }
         return nb;
     }
+    template <int MRT, bool ODD, bool WIDE>
+    static void staged_run(const KParams &p, void *A, const void *psi, const StagedSplit &sp, cudaStream_t st) {
+        const dim3 grid(sp.segments, (p.ny + sp.rows - 1) / sp.rows, (p.nzl + PLB_STAGED_ZC - 1) / PLB_STAGED_ZC);
+        if constexpr (Store<S>::SHIFT) {
+            if (p.stochastic) {
+                k_collide_staged<L, S, MRT, ODD, true, WIDE><<<grid, sp.threads, 0, st>>>(p, planes(p, A),
+                                                                                         (const float *)psi, sp);
+                return;
+            }
+        }
+        k_collide_staged<L, S, MRT, ODD, false, WIDE><<<grid, sp.threads, 0, st>>>(p, planes(p, A), (const float *)psi,
+                                                                                  sp);
+    }
     template <int MRT, bool ODD> static void collide_t(const KParams &p, void *A, const void *psi, cudaStream_t st) {
         dim3 grid, block;
         if constexpr (!std::is_same<S, double>::value) {
             if constexpr (std::is_same<L, D3Q19>::value) {
                 if (use_pair(p) && (std::is_same<S, __half>::value ? PLB_STAGED_HALF : PLB_STAGED_FLOAT) != 0) {
-                    constexpr int per = 2 * StagedShape<L>::THREADS;
-                    const dim3 sgrid((p.nx + per - 1) / per, p.ny, (p.nzl + PLB_STAGED_ZC - 1) / PLB_STAGED_ZC);
-                    const dim3 sblock(StagedShape<L>::THREADS);
-                    if constexpr (Store<S>::SHIFT) {
-                        if (p.stochastic) {
-                            k_collide_staged<L, S, MRT, ODD, true><<<sgrid, sblock, 0, st>>>(p, planes(p, A),
-                                                                                             (const float *)psi);
-                            return;
-                        }
-                    }
-                    k_collide_staged<L, S, MRT, ODD, false><<<sgrid, sblock, 0, st>>>(p, planes(p, A), (const float *)psi);
+                    bool wide = false;
+                    const StagedSplit sp = staged_split(p.nx / 2, p.ny, wide);
+                    if (wide) staged_run<MRT, ODD, true>(p, A, psi, sp, st);
+                    else staged_run<MRT, ODD, false>(p, A, psi, sp, st);
                     return;
                 }
             }

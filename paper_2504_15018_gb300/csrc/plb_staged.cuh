@@ -1,10 +1,10 @@
 // Fused force / collide / stream pass of the two-cell kernels with the populations of the
 // next plane staged in shared memory (cp.async) while the current plane is computed.
 //
-// A block of 64 threads owns a row segment of 128 cells (one cell pair per thread) and walks a
-// chunk of z planes.  For every plane it copies, per direction, the 64 aligned two-cell words
-// the threads read (plus one word on each side of the segment for the x-shifted reads of odd
-// steps, periodic wrap included, copied by ten lanes of the first warp, one x-shifted direction
+// A block owns a row segment of 64 cell pairs, or several rows or segments of up to 160 pairs in all
+// (staged_split), one pair per thread, and walks a chunk of z planes.  For every plane it copies, per
+// direction, the aligned two-cell words the threads read (plus one word on each side of a segment for
+// the x-shifted reads of odd steps, periodic wrap included, copied by ten lanes, one x-shifted direction
 // each) from global memory into one of two shared-memory buffers with asynchronous 4-byte
 // (FP16) or 8-byte (FP32) copies, one plane ahead of the computation, so the loads of plane
 // z + 1 are in flight while plane z is collided, without holding them in registers.  One
@@ -63,25 +63,53 @@ template <int N> __device__ __forceinline__ void cp_async_wait() {
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// Cell pairs of a row segment (threads of a block).
-#ifndef PLB_STAGED_THREADS
-#define PLB_STAGED_THREADS 64
-#endif
-
-template <class L> struct StagedShape {
-    static constexpr int THREADS = PLB_STAGED_THREADS;
-    static constexpr int WORDS = THREADS + 2;       // words staged per direction and plane
+// Shapes of a block: one row segment of 64 cell pairs, or (WIDE) up to 160 pairs of one or more whole
+// rows or row segments of equal width, in which a row width that is no multiple of 64 pairs leaves
+// fewer threads idle.  160 threads take as many registers per SM as 64-thread blocks do in all.
+template <bool WIDE> struct StagedShape {
+    static constexpr int THREADS = WIDE ? 160 : 64;
+    static constexpr int WORDS = WIDE ? 168 : 66;   // words staged per direction and plane: two more per row
 };
+
+// The rows and segments of a launch: blocks of `rows` rows, segments of `width` pairs.
+struct StagedSplit {
+    int width, rows, segments, threads;
+};
+
+// The split with the fewest threads, counting idle ones.  64 pairs of one row unless the wide shape
+// needs a tenth less (a row of 80 pairs took one full and one quarter-full block: now two rows are one
+// block of 160).  At least 128 threads, since the wide shape's shared memory allows eight blocks per SM,
+// and whole rows or 128-byte segments.  Step of 160^3 cells with stochastic rounding: 176 -> 136 us.
+inline StagedSplit staged_split(int pairs, int ny, bool &wide) {
+    StagedSplit best = {64, 1, (pairs + 63) / 64, 64};
+    double least = 0.9 * 64.0 * best.segments * ny;
+    wide = false;
+    for (int segments = 1; segments <= (pairs + 9) / 10 && segments <= 64; ++segments) {
+        const int width = (pairs + segments - 1) / segments;
+        if (width > StagedShape<true>::THREADS || width < 10) continue;      // (ten lanes per row copy the halo)
+        if ((pairs + width - 1) / width != segments || (segments > 1 && width < 32)) continue;
+        for (int rows = 1; rows <= ny && rows * width <= StagedShape<true>::THREADS; ++rows) {
+            if (rows * (width + 2) > StagedShape<true>::WORDS) break;
+            const int threads = (rows * width + 31) / 32 * 32;
+            const double all = (double)threads * segments * ((ny + rows - 1) / rows);
+            if (threads >= 128 && all < least) {
+                least = all;
+                best = {width, rows, segments, threads};
+                wide = true;
+            }
+        }
+    }
+    return best;
+}
 
 // Odd steps, D3Q19: the outer neighbour word of the segment for the k-th of the ten directions
 // with c_x != 0 (k < 10): x = X0 - 2 for c_x = +1, X0 + 2 nw for c_x = -1, periodic, from the
 // source row of the direction (y - c_y, z - c_z).  Directions 1, 2 (x axis), 7-10 (x-y edges),
 // 11-14 (x-z edges); odd i has c_x = +1, and c_y (7-10) or c_z (11-14) is +1, -1, -1, +1.
-template <class S, bool WALL>
+template <class S, bool WALL, int NW>
 __device__ __forceinline__ void stage_halo_d3q19(const KParams &p, const Planes<S> &A, typename StageWord<S>::W *buf,
                                                  int X0, int nw, int k, int y, int z) {
     using SW = StageWord<S>;
-    constexpr int NW = StagedShape<D3Q19>::WORDS;
     const int i = k < 2 ? 1 + k : 5 + k;
     const int o = (i & 1) ? i + 1 : i - 1;
     const int m = (i - 7) & 3;
@@ -99,16 +127,17 @@ __device__ __forceinline__ void stage_halo_d3q19(const KParams &p, const Planes<
         SW::copy(buf + i * NW + nw + 1, elem(A.p[o], r + (X0 + 2 * nw < p.nx ? X0 + 2 * nw : 0)));
 }
 
-// Copies plane z's words of every direction into buf.  x0 = X0 + 2 t; nw: active threads of
-// the segment; active: this thread's pair lies in the lattice.
-template <class L, class S, bool ODD, bool WALL>
+// Copies plane z's words of every direction into buf (this thread's row).  The thread's pair is pair t of
+// the nw that its segment has in row y; lane < 10: it also copies that outer word of row hy, whose words
+// are at hbuf.
+template <class L, class S, bool ODD, bool WALL, int NW>
 __device__ __forceinline__ void stage_plane(const KParams &p, const Planes<S> &A, typename StageWord<S>::W *buf,
-                                            int X0, int nw, int t, int y, int z) {
+                                            typename StageWord<S>::W *hbuf, int X0, int nw, int t, int y, int hy,
+                                            int lane, int z) {
     using SW = StageWord<S>;
-    constexpr int NW = StagedShape<L>::WORDS;
     // the segment's outer words of the ten x-shifted directions, one lane each
     static_assert(std::is_same<L, D3Q19>::value, "staged kernel: D3Q19 directions");
-    if (ODD && t < 10) stage_halo_d3q19<S, WALL>(p, A, buf, X0, nw, t, y, z);
+    if (ODD && lane < 10) stage_halo_d3q19<S, WALL, NW>(p, A, hbuf, X0, nw, lane, hy, z);
     if (t >= nw) return;
     GeoPair g;
     geo_pair_at(p, X0 + 2 * t, y, z, g);
@@ -129,11 +158,10 @@ __device__ __forceinline__ void stage_plane(const KParams &p, const Planes<S> &A
 }
 
 // The two cells' pre-collision populations from the staged buffer.
-template <class L, class S, bool ODD, bool WALL>
+template <class L, class S, bool ODD, bool WALL, int NW>
 __device__ __forceinline__ void read_staged(const KParams &p, const typename StageWord<S>::W *buf, int t, int y,
                                             f2 *f) {
     using SW = StageWord<S>;
-    constexpr int NW = StagedShape<L>::WORDS;
     Unroll<0, L::Q>::run([&](auto ic) {
         constexpr int i = decltype(ic)::value;
         constexpr int cx = L::cx(i), cy = L::cy(i);
@@ -150,12 +178,27 @@ __device__ __forceinline__ void read_staged(const KParams &p, const typename Sta
     });
 }
 
-template <class L, class S, int MRT, bool ODD, bool WALL, bool SR>
+template <class L, class S, int MRT, bool ODD, bool WALL, bool SR, bool WIDE>
 __device__ __forceinline__ void staged_walk(const KParams &p, const Planes<S> &A, const float *__restrict__ psi,
-                                            typename StageWord<S>::W (*stage)[L::Q * StagedShape<L>::WORDS]) {
-    const int t = threadIdx.x, X0 = blockIdx.x * (2 * StagedShape<L>::THREADS), y = blockIdx.y;
+                                            typename StageWord<S>::W (*stage)[L::Q * StagedShape<WIDE>::WORDS],
+                                            const StagedSplit &sp) {
+    constexpr int NW = StagedShape<WIDE>::WORDS;
+    // row and pair of this thread, and the row whose outer words it copies (idle threads: t = nw)
+    const int row = WIDE ? (int)threadIdx.x / sp.width : 0;
+    const int width = WIDE ? sp.width : StagedShape<WIDE>::THREADS;
+    const int X0 = blockIdx.x * (2 * width), y0 = WIDE ? blockIdx.y * sp.rows : blockIdx.y, y = y0 + row;
     const int rem = (p.nx - X0) / 2;
-    const int nw = rem < StagedShape<L>::THREADS ? rem : StagedShape<L>::THREADS;
+    const int nw = rem < width ? rem : width;
+    int t = threadIdx.x - row * width;
+    int lane = threadIdx.x, hy = y0, hrow = 0;
+    if (WIDE) {
+        if (row >= sp.rows || y >= p.ny) t = nw;
+        hrow = lane / 10;
+        lane -= 10 * hrow;
+        hy = y0 + hrow;
+        if (hrow >= sp.rows || hy >= p.ny) lane = 10;
+    }
+    const int at = row * (width + 2), hat = hrow * (width + 2);
     const int zb = p.z0 + blockIdx.z * PLB_STAGED_ZC;
     const int zlim = p.z0 + p.nzl;
     const int ze = zb + PLB_STAGED_ZC < zlim ? zb + PLB_STAGED_ZC : zlim;
@@ -163,7 +206,8 @@ __device__ __forceinline__ void staged_walk(const KParams &p, const Planes<S> &A
     constexpr int NB = PLB_STAGED_BUFS;
 #pragma unroll
     for (int j = 0; j < NB - 1; ++j) {
-        if (zb + j < ze) stage_plane<L, S, ODD, WALL>(p, A, stage[j], X0, nw, t, y, zb + j);
+        if (zb + j < ze)
+            stage_plane<L, S, ODD, WALL, NW>(p, A, stage[j] + at, stage[j] + hat, X0, nw, t, y, hy, lane, zb + j);
         cp_async_commit();
     }
     int cur = 0;                                   // buffer of plane z
@@ -173,11 +217,13 @@ __device__ __forceinline__ void staged_walk(const KParams &p, const Planes<S> &A
         cp_async_wait<NB - 2>();
         __syncthreads();
         const int nxt = cur == 0 ? NB - 1 : cur - 1;   // (cur + NB - 1) mod NB: plane z - 1's buffer
-        if (z + NB - 1 < ze) stage_plane<L, S, ODD, WALL>(p, A, stage[nxt], X0, nw, t, y, z + NB - 1);
+        if (z + NB - 1 < ze)
+            stage_plane<L, S, ODD, WALL, NW>(p, A, stage[nxt] + at, stage[nxt] + hat, X0, nw, t, y, hy, lane,
+                                             z + NB - 1);
         cp_async_commit();
         if (t < nw) {
             f2 f[L::Q];
-            read_staged<L, S, ODD, WALL>(p, stage[cur], t, y, f);
+            read_staged<L, S, ODD, WALL, NW>(p, stage[cur] + at, t, y, f);
             GeoPair g;
             geo_pair_at(p, X0 + 2 * t, y, z, g);
             f2 F[3];
@@ -200,14 +246,14 @@ __device__ __forceinline__ void staged_walk(const KParams &p, const Planes<S> &A
 #define PLB_STAGED_MAXREG_SR 84
 #endif
 
-template <class L, class S, int MRT, bool ODD, bool SR>
-__global__ void __maxnreg__(SR ? PLB_STAGED_MAXREG_SR : PLB_STAGED_MAXREG) k_collide_staged(KParams p, Planes<S> A, const float *__restrict__ psi) {
-    __shared__ __align__(16) typename StageWord<S>::W stage[PLB_STAGED_BUFS][L::Q * StagedShape<L>::WORDS];
-    const int y = blockIdx.y;
-    if (ODD && p.wall_y && (y == 0 || y == p.ny - 1))
-        staged_walk<L, S, MRT, ODD, true, SR>(p, A, psi, stage);
+template <class L, class S, int MRT, bool ODD, bool SR, bool WIDE>
+__global__ void __maxnreg__(SR ? PLB_STAGED_MAXREG_SR : PLB_STAGED_MAXREG) k_collide_staged(KParams p, Planes<S> A, const float *__restrict__ psi, StagedSplit sp) {
+    __shared__ __align__(16) typename StageWord<S>::W stage[PLB_STAGED_BUFS][L::Q * StagedShape<WIDE>::WORDS];
+    const int y0 = WIDE ? blockIdx.y * sp.rows : blockIdx.y, y1 = WIDE ? y0 + sp.rows : y0 + 1;
+    if (ODD && p.wall_y && (y0 == 0 || y1 >= p.ny))
+        staged_walk<L, S, MRT, ODD, true, SR, WIDE>(p, A, psi, stage, sp);
     else
-        staged_walk<L, S, MRT, ODD, false, SR>(p, A, psi, stage);
+        staged_walk<L, S, MRT, ODD, false, SR, WIDE>(p, A, psi, stage, sp);
 }
 
 }  // namespace plb
