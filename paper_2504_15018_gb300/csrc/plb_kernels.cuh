@@ -501,6 +501,21 @@ template <class L, class S> struct Launch {
                      cudaStream_t st) {
         k_init<L, S><<<blocks(cn, 256), 256, 0, st>>>(p, (S *)A, rho0, u0, c0, cn, u0 != nullptr);
     }
+    // Launches a step kernel so that it may start while the kernel before it in the stream runs out
+    // (step_kernel_begin waits for that one).
+    template <class... P, class... Args>
+    static void go(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, const Args &...args) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = grid;
+        cfg.blockDim = block;
+        cfg.stream = st;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+    }
     static Planes<S> planes(const KParams &p, const void *A) {
         Planes<S> pl;
         for (int i = 0; i < 19; ++i) pl.p[i] = (S *)A + (i < L::Q ? (long long)i * p.pstride : 0);
@@ -534,22 +549,22 @@ template <class L, class S> struct Launch {
         if constexpr (std::is_same<S, __half>::value) {
             if (PLB_PSI_QUAD && p.nx % 4 == 0 && p.n < (1LL << 31)) {
                 const long long quads = (long long)(p.nx / 4) * p.ny;
-                k_psi_quad<L, ODD><<<dim3(blocks(quads, 256), 1, p.nzl), 256, 0, st>>>(p, planes(p, A), (float *)psi);
+                go(k_psi_quad<L, ODD>, dim3(blocks(quads, 256), 1, p.nzl), 256, st, p, planes(p, A), (float *)psi);
                 return;
             }
         }
         if constexpr (!std::is_same<S, double>::value) {
             if (use_pair(p)) {
                 dims_pair(p, grid, block);
-                k_psi_pair<L, S, ODD><<<grid, block, 0, st>>>(p, planes(p, A), (float *)psi);
+                go(k_psi_pair<L, S, ODD>, grid, block, st, p, planes(p, A), (float *)psi);
                 return;
             }
         }
         dims3(p, grid, block);
         if (p.n < (1LL << 31))
-            k_psi_fast<L, S, ODD, int><<<grid, block, 0, st>>>(p, planes(p, A), (PsiT *)psi);
+            go(k_psi_fast<L, S, ODD, int>, grid, block, st, p, planes(p, A), (PsiT *)psi);
         else
-            k_psi_fast<L, S, ODD, long long><<<grid, block, 0, st>>>(p, planes(p, A), (PsiT *)psi);
+            go(k_psi_fast<L, S, ODD, long long>, grid, block, st, p, planes(p, A), (PsiT *)psi);
     }
     static void psi(const KParams &p, const void *A, void *psi, int odd, cudaStream_t st) {
         if (odd) psi_t<true>(p, A, psi, st);
@@ -572,13 +587,12 @@ template <class L, class S> struct Launch {
         const dim3 grid(sp.segments, (p.ny + sp.rows - 1) / sp.rows, (p.nzl + PLB_STAGED_ZC - 1) / PLB_STAGED_ZC);
         if constexpr (Store<S>::SHIFT) {
             if (p.stochastic) {
-                k_collide_staged<L, S, MRT, ODD, true, WIDE><<<grid, sp.threads, 0, st>>>(p, planes(p, A),
-                                                                                         (const float *)psi, sp);
+                go(k_collide_staged<L, S, MRT, ODD, true, WIDE>, grid, sp.threads, st, p, planes(p, A),
+                   (const float *)psi, sp);
                 return;
             }
         }
-        k_collide_staged<L, S, MRT, ODD, false, WIDE><<<grid, sp.threads, 0, st>>>(p, planes(p, A), (const float *)psi,
-                                                                                  sp);
+        go(k_collide_staged<L, S, MRT, ODD, false, WIDE>, grid, sp.threads, st, p, planes(p, A), (const float *)psi, sp);
     }
     template <int MRT, bool ODD> static void collide_t(const KParams &p, void *A, const void *psi, cudaStream_t st) {
         dim3 grid, block;
@@ -607,28 +621,27 @@ template <class L, class S> struct Launch {
                 }
                 if constexpr (Store<S>::SHIFT) {
                     if (p.stochastic) {
-                        k_collide_pair<L, S, MRT, ODD, true><<<grid, block, 0, st>>>(q, planes(p, A),
-                                                                                    (const float *)psi);
+                        go(k_collide_pair<L, S, MRT, ODD, true>, grid, block, st, q, planes(p, A), (const float *)psi);
                         return;
                     }
                 }
-                k_collide_pair<L, S, MRT, ODD, false><<<grid, block, 0, st>>>(q, planes(p, A), (const float *)psi);
+                go(k_collide_pair<L, S, MRT, ODD, false>, grid, block, st, q, planes(p, A), (const float *)psi);
                 return;
             }
         }
         if constexpr (std::is_same<S, double>::value) {
             dims3(p, grid, block, 128);
             if (p.n < (1LL << 31))
-                k_collide_plain<L, MRT, ODD, int><<<grid, block, 0, st>>>(p, planes(p, A), (const double *)psi);
+                go(k_collide_plain<L, MRT, ODD, int>, grid, block, st, p, planes(p, A), (const double *)psi);
             else
-                k_collide_plain<L, MRT, ODD, long long><<<grid, block, 0, st>>>(p, planes(p, A), (const double *)psi);
+                go(k_collide_plain<L, MRT, ODD, long long>, grid, block, st, p, planes(p, A), (const double *)psi);
             return;
         }
         dims3(p, grid, block);
         if (p.n < (1LL << 31))
-            k_collide_fast<L, S, MRT, ODD, int><<<grid, block, 0, st>>>(p, planes(p, A), (const PsiT *)psi);
+            go(k_collide_fast<L, S, MRT, ODD, int>, grid, block, st, p, planes(p, A), (const PsiT *)psi);
         else
-            k_collide_fast<L, S, MRT, ODD, long long><<<grid, block, 0, st>>>(p, planes(p, A), (const PsiT *)psi);
+            go(k_collide_fast<L, S, MRT, ODD, long long>, grid, block, st, p, planes(p, A), (const PsiT *)psi);
     }
     static void collide_bgk(const KParams &p, void *A, const void *psi, int odd, cudaStream_t st) {
         if (odd) collide_t<0, true>(p, A, psi, st);

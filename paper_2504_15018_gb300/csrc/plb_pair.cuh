@@ -363,6 +363,7 @@ __device__ __forceinline__ void psi_pair_body(const KParams &p, const Planes<S> 
 
 template <class L, class S, bool ODD>
 __global__ void __launch_bounds__(256) k_psi_pair(KParams p, Planes<S> A, float *__restrict__ psi) {
+    step_kernel_begin();
     GeoPair g;
     if (!make_geo_pair(p, g)) return;
     if (ODD && p.wall_y && (g.y == 0 || g.y == p.ny - 1))
@@ -437,6 +438,7 @@ __device__ __forceinline__ void psi_quad_body(const KParams &p, const Planes<__h
 // against 32 / 44 with the thread count alone), measured 92.9 -> 94.2 % of the copy bandwidth.
 template <class L, bool ODD>
 __global__ void __launch_bounds__(256, 1) k_psi_quad(KParams p, Planes<__half> A, float *__restrict__ psi) {
+    step_kernel_begin();
     // a plane's quads in one row of blocks: rows that are no multiple of a block leave no threads idle
     const int q = blockIdx.x * blockDim.x + threadIdx.x, nq = p.nx / 4, y = q / nq, x0 = 4 * (q - y * nq);
     if (y >= p.ny) return;
@@ -490,6 +492,7 @@ __device__ __forceinline__ void prefetch_ahead_pair(const KParams &p, const Plan
 // round-to-nearest kernel is register-allocated for its own path.
 template <class L, class S, int MRT, bool ODD, bool SR>
 __global__ void __maxnreg__(PLB_PAIR_MAXREG) k_collide_pair(KParams p, Planes<S> A, const float *__restrict__ psi) {
+    step_kernel_begin();
     if (p.prefetch_ahead > 0) prefetch_ahead_pair<L, S>(p, A);
     GeoPair g;
     if (!make_geo_pair(p, g)) return;

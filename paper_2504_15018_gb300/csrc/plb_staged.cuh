@@ -248,6 +248,7 @@ __device__ __forceinline__ void staged_walk(const KParams &p, const Planes<S> &A
 
 template <class L, class S, int MRT, bool ODD, bool SR, bool WIDE>
 __global__ void __maxnreg__(SR ? PLB_STAGED_MAXREG_SR : PLB_STAGED_MAXREG) k_collide_staged(KParams p, Planes<S> A, const float *__restrict__ psi, StagedSplit sp) {
+    step_kernel_begin();
     __shared__ __align__(16) typename StageWord<S>::W stage[PLB_STAGED_BUFS][L::Q * StagedShape<WIDE>::WORDS];
     const int y0 = WIDE ? blockIdx.y * sp.rows : blockIdx.y, y1 = WIDE ? y0 + sp.rows : y0 + 1;
     if (ODD && p.wall_y && (y0 == 0 || y1 >= p.ny))

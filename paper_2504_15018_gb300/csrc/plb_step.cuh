@@ -543,6 +543,7 @@ __device__ __forceinline__ void psi_body(const KParams &p, const Planes<S> &A, t
 
 template <class L, class S, bool ODD, class I>
 __global__ void __launch_bounds__(256) k_psi_fast(KParams p, Planes<S> A, typename Store<S>::PsiT *__restrict__ psi) {
+    step_kernel_begin();
     Geo<I> g;
     if (!make_geo<I>(p, g)) return;
     if (ODD && p.wall_y && (g.y == 0 || g.y == p.ny - 1))
@@ -575,6 +576,7 @@ __device__ __forceinline__ void collide_body(const KParams &p, const Planes<S> &
 // without a residency floor on the register allocation.
 template <class L, int MRT, bool ODD, class I>
 __global__ void __launch_bounds__(128) k_collide_plain(KParams p, Planes<double> A, const double *__restrict__ psi) {
+    step_kernel_begin();
     Geo<I> g;
     if (!make_geo<I>(p, g)) return;
     if (ODD && p.wall_y && (g.y == 0 || g.y == p.ny - 1))
@@ -586,6 +588,7 @@ __global__ void __launch_bounds__(128) k_collide_plain(KParams p, Planes<double>
 template <class L, class S, int MRT, bool ODD, class I>
 __global__ void __launch_bounds__(256, PLB_COLLIDE_MINB) k_collide_fast(KParams p, Planes<S> A,
                                                       const typename Store<S>::PsiT *__restrict__ psi) {
+    step_kernel_begin();
     Geo<I> g;
     if (!make_geo<I>(p, g)) return;
     const bool wall = ODD && p.wall_y && (g.y == 0 || g.y == p.ny - 1);
