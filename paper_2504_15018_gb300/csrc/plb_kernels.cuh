@@ -229,7 +229,7 @@ __global__ void k_set_pops(KParams p, S *__restrict__ A, const double *__restric
 // population in FP64 took about 100 of them per cell, ten times the HBM time.  FP32 storage adds with
 // error-free transformations on the FP32 pipe instead and converts once per thread; the speed
 // maximum is searched in pairs of FP32 values, and FP64 evaluates the candidates only.  Mass, momentum,
-// maximum speed and moments of 256 x 128 x 128 cells, D3Q19 FP32: 2140 -> 800 us.
+// maximum speed and moments of 256 x 128 x 128 cells, D3Q19 FP32: 2140 -> 706 us.
 
 // A sum of FP32 values in three FP32 parts, each the rounding error of the one before (TwoSum, Knuth
 // 1969; the cascade of Ogita, Rump and Oishi 2005): about 70 bits, where FP64 keeps 53.
@@ -369,9 +369,11 @@ __global__ void __launch_bounds__(256) k_reduce(KParams p, const S *__restrict__
     block_partial(acc, what == 2, partials);
 }
 
-// FP32 arithmetic: density (WHAT 0), momentum (1) and the largest speed (2).
+// FP32 arithmetic: density (WHAT 0), momentum (1) and the largest speed (2).  Four blocks per SM: at the
+// 128 registers that it takes uncapped, two, a long chain of additions per cell has too little beside it
+// (the four readouts of 256 x 128 x 128 cells, two / three / four / five blocks: 805 / 719 / 706 / 731 us).
 template <class L, class S, int WHAT>
-__global__ void __launch_bounds__(256) k_reduce_f32(KParams p, const S *__restrict__ A, const float *__restrict__ psi,
+__global__ void __launch_bounds__(256, 4) k_reduce_f32(KParams p, const S *__restrict__ A, const float *__restrict__ psi,
                                                     int odd, Box box, double *__restrict__ partials) {
     double acc[4] = {0, 0, 0, 0};
     Sum3 sum[3];
