@@ -40,26 +40,27 @@ __device__ __forceinline__ int wrap_near(int v, int n) {
     return v;
 }
 
-// Tile rows (FP32 and FP16 storage) and threads per block of the single pass (two blocks of 256
-// threads per SM at the 128-register cap).  D3Q19 plates workload, GLUPS with 8 / 16 / 32 rows:
-// FP32 27.9 / 29.0 / 26.6, FP16S 31.7 / 34.3 / 36.2.
+// Tile rows and threads per block, at the 128-register cap (512 threads per SM).  D3Q19 FP32: four blocks
+// of 128 threads and 8 rows; a block's psi and collision phases are apart, so more and smaller blocks
+// overlap loads with arithmetic better, which is worth more than their larger halo.  Milliseconds a step
+// with 16 rows x 256 threads and now: 512 x 256 x 256 1.156 and 1.126, 394 x 250 x 186 0.750 and 0.709,
+// 96 x 100 x 90 0.053 and 0.043 (64 x 4 rows: 1.156, 0.718, 0.046; 128 x 12: 1.184, 0.749, 0.047).  FP16
+// (32 rows) and D2Q9 (16 rows) keep 256 threads.
 #ifndef PLB_FUSED_TY
-#define PLB_FUSED_TY 16
-#endif
-#ifndef PLB_FUSED_TY_HALF
-#define PLB_FUSED_TY_HALF 32
+#define PLB_FUSED_TY 8
 #endif
 #ifndef PLB_FUSED_THREADS
-#define PLB_FUSED_THREADS 256
+#define PLB_FUSED_THREADS 128
 #endif
 
 template <class L, class S> struct FusedTile {
+    static constexpr bool SMALL = L::D == 3 && sizeof(S) == 4;
     static constexpr int TX = 64;                      // cells in x (32 pairs)
-    static constexpr int TY = sizeof(S) == 2 ? PLB_FUSED_TY_HALF : PLB_FUSED_TY;   // rows
+    static constexpr int TY = SMALL ? PLB_FUSED_TY : (sizeof(S) == 2 ? 32 : 16);   // rows
     static constexpr int HP = TX / 2 + 2;              // pairs per shared row: one halo pair each side
     static constexpr int RY = TY + 2;                  // rows with the halo
     static constexpr int NPL = L::D == 3 ? 3 : 1;      // psi planes in the ring
-    static constexpr int THREADS = PLB_FUSED_THREADS;
+    static constexpr int THREADS = SMALL ? PLB_FUSED_THREADS : 256;
 };
 
 // psi of the halo-extended tile of plane zg (any integer: wrapped) into ring plane `plane`.
@@ -137,7 +138,8 @@ __device__ __forceinline__ void fused_collide_plane(const KParams &p, const Plan
 
 // Grid: (ceil(nx / TX), ceil(ny / TY), ceil(nz / zc)); block: THREADS threads.
 template <class L, class S, int MRT, bool SR>
-__global__ void __launch_bounds__(PLB_FUSED_THREADS, 512 / PLB_FUSED_THREADS) k_fused_pair(KParams p, Planes<S> A, Planes<S> B, int zc) {
+__global__ void __launch_bounds__((FusedTile<L, S>::THREADS), (512 / FusedTile<L, S>::THREADS))
+    k_fused_pair(KParams p, Planes<S> A, Planes<S> B, int zc) {
     using Tl = FusedTile<L, S>;
     constexpr int PLANE = Tl::RY * 2 * Tl::HP;
     __shared__ __align__(16) float ring[Tl::NPL * PLANE];
