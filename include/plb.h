@@ -233,8 +233,9 @@ int plb_si_convert(const double si[6], const double lat[3], double xi, double ou
  * EOS, tau, eps, kappa, walls and forces may differ per instance) advanced together by one
  * persistent kernel launch per plb_batch_step call: every step is a psi pass over all
  * instances, a grid barrier, the fused force/collide/stream pass, and another barrier
- * (the same per-cell update as plb_step, Sec. II of the paper).  Work is split into tiles of
- * whole rows; the tile size and resident blocks per SM are set by plb_batch_autotune or
+ * (the same per-cell update as plb_step, Sec. II of the paper).  A batch larger than the L2
+ * cache is stepped in groups of instances, one after the other, each for all nsteps.  Work is
+ * split into tiles; the tile size and resident blocks per SM are set by plb_batch_autotune or
  * plb_batch_configure.  The grid barrier waits a bounded time: a wait that runs out sets a
  * device error word, the kernel returns, and plb_batch_status reports PLB_ETIMEOUT. */
 typedef struct plb_batch_state plb_batch_t;
@@ -275,7 +276,7 @@ int plb_batch_status(plb_batch_t *b);
 /* Clears a recorded barrier timeout. */
 int plb_batch_reset_error(plb_batch_t *b);
 
-/* Tile size in cells (rows of a tile = tile_cells / nx, at least 1), resident 256-thread
+/* Tile size in cells (no less than a row or 256 threads' cells), resident 256-thread
  * blocks per SM, and the barrier's polling limit (0 keeps the default, about a second or more).
  * A non-positive tile_cells or blocks_per_sm keeps the current value. */
 int plb_batch_configure(plb_batch_t *b, int tile_cells, int blocks_per_sm, unsigned spin_limit);

@@ -1,6 +1,7 @@
 // Persistent kernel of a batch of independent lattices: every step runs the psi pass over
-// all tiles of all instances, a grid barrier, the fused force/collide/stream pass, and a
-// second barrier, for nsteps steps in one launch.  Loads follow LdBatch (populations through
+// all tiles of its instances, a grid barrier, the fused force/collide/stream pass, and a
+// second barrier, for nsteps steps in one launch (a batch larger than L2: one group of instances after
+// the other, each for all steps).  Loads follow LdBatch (populations through
 // L2 only, the psi stencil through L1 after the barrier's acquire):
 // blocks read, across barriers, what other SMs wrote in the same launch.
 #pragma once
@@ -35,7 +36,7 @@ __device__ __forceinline__ bool grid_sync(GridBar *bar, unsigned expected, unsig
                     atomicOr(&bar->err, 1u);
                     break;
                 }
-                __nanosleep(256);
+                __nanosleep(64);
             }
         }
         __threadfence();
@@ -50,10 +51,8 @@ __device__ __forceinline__ void batch_tile(const BatchInst &in, const BatchTile 
     const KParams &p = in.kp;
     const Planes<S> &A = *reinterpret_cast<const Planes<S> *>(in.pl);
     using PsiT = typename Store<S>::PsiT;
-    const int units = (tl.y1 - tl.y0) * in.upr;
-    for (int j = threadIdx.x; j < units; j += blockDim.x) {
-        const int r = j / in.upr;
-        const int y = tl.y0 + r, xu = j - r * in.upr;
+    for (int u = tl.u0 + threadIdx.x; u < tl.u1; u += blockDim.x) {
+        const int y = u / in.upr, xu = u - y * in.upr;
         const bool wall = odd && p.wall_y && (y == 0 || y == p.ny - 1);
         bool done = false;
         if constexpr (!std::is_same<S, double>::value) {
@@ -90,29 +89,60 @@ __device__ __forceinline__ void batch_tile(const BatchInst &in, const BatchTile 
     }
 }
 
+// Instance descriptors that a block keeps in shared memory: its tiles are consecutive, so they belong to
+// few instances, and parameters read from shared memory replace about 60 loads per cell from global
+// memory, which the barriers' acquires drop from L1.
+constexpr int kBatchWindow = 4;
+
 template <class L, class S, int MRT>
 __global__ void __launch_bounds__(256, BatchMinBlocks<L>::value) k_batch(BatchLaunch b) {
+    __shared__ BatchInst window[kBatchWindow];
     const unsigned salt0 = *reinterpret_cast<volatile unsigned *>(&b.bar->salt);
-    for (int step = 0; step < b.nsteps; ++step) {
-        for (int t = blockIdx.x; t < b.ntiles; t += gridDim.x) {
-            const BatchTile tl = b.tiles[t];
-            const BatchInst &in = b.insts[tl.inst];
-            batch_tile<L, S, MRT, true, false>(in, tl, (in.odd + step) & 1, 0);
+    int held = -1;                                // first instance in the window (the same in all threads)
+    auto instance = [&](int k) -> const BatchInst & {
+        if (held < 0 || k < held || k >= held + kBatchWindow) {
+            static_assert(sizeof(BatchInst) % 8 == 0, "copied in 8-byte words");
+            __syncthreads();
+            held = k;
+            const int n = b.ninst - k < kBatchWindow ? b.ninst - k : kBatchWindow;
+            const unsigned long long *src = reinterpret_cast<const unsigned long long *>(b.insts + k);
+            unsigned long long *dst = reinterpret_cast<unsigned long long *>(window);
+            for (int w = threadIdx.x; w < n * (int)(sizeof(BatchInst) / 8); w += blockDim.x) dst[w] = src[w];
+            __syncthreads();
         }
-        if (!grid_sync(b.bar, b.expected, b.spin_limit)) return;
-        for (int t = blockIdx.x; t < b.ntiles; t += gridDim.x) {
-            const BatchTile tl = b.tiles[t];
-            const BatchInst &in = b.insts[tl.inst];
-            const int odd = (in.odd + step) & 1;
-            if constexpr (Store<S>::SHIFT) {
-                if (in.kp.stochastic) {
-                    batch_tile<L, S, MRT, false, true>(in, tl, odd, salt0 + step);
-                    continue;
-                }
+        // (through a pointer of unknown origin: knowing that no store changes the window, the compiler
+        // loads all parameters up front and spills 90 bytes)
+        const BatchInst *in = window + (k - held);
+        asm("" : "+l"(in));
+        return *in;
+    };
+    // group by group, each for all steps; in a group, consecutive tiles, the same number (give or take one)
+    // for every block
+    for (int group = 0; group < b.ngroups; ++group) {
+        const int g0 = b.groups[group], gn = b.groups[group + 1] - g0;
+        const int t0 = g0 + (int)((long long)gn * blockIdx.x / gridDim.x);
+        const int t1 = g0 + (int)((long long)gn * (blockIdx.x + 1) / gridDim.x);
+        for (int step = 0; step < b.nsteps; ++step) {
+            for (int t = t0; t < t1; ++t) {
+                const BatchTile tl = b.tiles[t];
+                const BatchInst &in = instance(tl.inst);
+                batch_tile<L, S, MRT, true, false>(in, tl, (in.odd + step) & 1, 0);
             }
-            batch_tile<L, S, MRT, false, false>(in, tl, odd, 0);
+            if (!grid_sync(b.bar, b.expected, b.spin_limit)) return;
+            for (int t = t0; t < t1; ++t) {
+                const BatchTile tl = b.tiles[t];
+                const BatchInst &in = instance(tl.inst);
+                const int odd = (in.odd + step) & 1;
+                if constexpr (Store<S>::SHIFT) {
+                    if (in.kp.stochastic) {
+                        batch_tile<L, S, MRT, false, true>(in, tl, odd, salt0 + step);
+                        continue;
+                    }
+                }
+                batch_tile<L, S, MRT, false, false>(in, tl, odd, 0);
+            }
+            if (!grid_sync(b.bar, b.expected, b.spin_limit)) return;
         }
-        if (!grid_sync(b.bar, b.expected, b.spin_limit)) return;
     }
     // every block has passed the last barrier: advance the stored parities and the step salt
     if (blockIdx.x == 0) {

@@ -80,9 +80,9 @@ struct BatchInst {
     int upr;               // work units per row: nx / 2 (pair) or nx
     int pad;
 };
-// A tile: rows y0 <= y < y1 of plane z of one instance.
+// A tile: work units u0 <= u < u1 (x fastest) of plane z of one instance.
 struct BatchTile {
-    int inst, z, y0, y1;
+    int inst, z, u0, u1;
 };
 // Grid barrier state (device memory, zeroed at creation).
 struct GridBar {
@@ -92,7 +92,8 @@ struct GridBar {
 struct BatchLaunch {
     BatchInst *insts;
     const BatchTile *tiles;
-    int ninst, ntiles, nsteps;
+    const int *groups;       // first tile of each group of instances, and the number of tiles
+    int ninst, ngroups, nsteps;
     GridBar *bar;
     unsigned spin_limit;     // bounded wait: polls of the barrier before giving up
     unsigned expected;       // blocks the barrier waits for (gridDim.x unless testing a timeout)
