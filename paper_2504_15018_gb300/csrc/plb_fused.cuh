@@ -40,12 +40,13 @@ __device__ __forceinline__ int wrap_near(int v, int n) {
     return v;
 }
 
-// Tile rows and threads per block, at the 128-register cap (512 threads per SM).  D3Q19 FP32: four blocks
-// of 128 threads and 8 rows; a block's psi and collision phases are apart, so more and smaller blocks
-// overlap loads with arithmetic better, which is worth more than their larger halo.  Milliseconds a step
-// with 16 rows x 256 threads and now: 512 x 256 x 256 1.156 and 1.126, 394 x 250 x 186 0.750 and 0.709,
-// 96 x 100 x 90 0.053 and 0.043 (64 x 4 rows: 1.156, 0.718, 0.046; 128 x 12: 1.184, 0.749, 0.047).  FP16
-// (32 rows) and D2Q9 (16 rows) keep 256 threads.
+// Tile rows and threads per block, at the 128-register cap (512 threads per SM).  D3Q19: four blocks of 128
+// threads and 8 rows; a block's psi and collision phases are apart, so more and smaller blocks overlap
+// loads with arithmetic better, which is worth more than their larger halo.  Milliseconds a step with 256
+// threads (16 rows FP32, 32 FP16) and now: FP32 512 x 256 x 256 1.156 and 1.126, 394 x 250 x 186 0.750 and
+// 0.709, 96 x 100 x 90 0.053 and 0.043 (64 x 4 rows: 1.156, 0.718, 0.046; 128 x 12: 1.184, 0.749, 0.047);
+// FP16 0.921 and 0.879, 0.592 and 0.560, with stochastic rounding 0.066 and 0.046 (128 x 16: 0.902, 0.557,
+// 0.054).  D2Q9, without a second phase to overlap, runs the same with 8 to 24 rows: 256 threads.
 #ifndef PLB_FUSED_TY
 #define PLB_FUSED_TY 8
 #endif
@@ -54,7 +55,7 @@ __device__ __forceinline__ int wrap_near(int v, int n) {
 #endif
 
 template <class L, class S> struct FusedTile {
-    static constexpr bool SMALL = L::D == 3 && sizeof(S) == 4;
+    static constexpr bool SMALL = L::D == 3;
     static constexpr int TX = 64;                      // cells in x (32 pairs)
     static constexpr int TY = SMALL ? PLB_FUSED_TY : (sizeof(S) == 2 ? 32 : 16);   // rows
     static constexpr int HP = TX / 2 + 2;              // pairs per shared row: one halo pair each side
