@@ -256,28 +256,40 @@ struct Sum3 {
     }
 };
 
-// |momentum|^2 / rho^2 (scaled by 2^60) as a pair of FP32 values, relative error below 2^-40.
-__device__ __forceinline__ void speed2_pair(const Sum3 &rho, const Sum3 m[3], int dims, float &qh, float &ql) {
-    float nh = 0.0f, nl = 0.0f, e;
+// speed^2 = |momentum|^2 / rho^2 of a cell as a pair of FP32 values, relative error below 2^-40: true where the
+// pair says so.  Density and momentum are scaled by the power of two that brings the density to 1 .. 2
+// (exact), so that no square leaves FP32's range for any density as long as the speed lies in 2^-45 .. 2^50.
+// False for every other cell (its rounding errors could be subnormal, its squares overflow, or its density
+// is 0, infinite or NaN).  A cell without momentum has speed 0.
+__device__ __forceinline__ bool speed2_pair(const Sum3 &rho, const Sum3 m[3], int dims, float &qh, float &ql) {
+    float rh, rl;
+    rho.pair(rh, rl);
+    int e = (int)(__float_as_uint(rh) >> 23 & 0xffu);
+    e = e < 1 ? 1 : (e > 253 ? 253 : e);
+    const float scale = __uint_as_float((unsigned)(254 - e) << 23);        // 2^(127 - e)
+    rh = __fmul_rn(rh, scale);
+    rl = __fmul_rn(rl, scale);
+    float nh = 0.0f, nl = 0.0f, err;
+    bool still = true;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         if (a >= dims) continue;
         float h, l;
         m[a].pair(h, l);
-        h = __fmul_rn(h, 0x1p30f);
-        l = __fmul_rn(l, 0x1p30f);
+        still = still && h == 0.0f;
+        h = __fmul_rn(h, scale);
+        l = __fmul_rn(l, scale);
         const float s = __fmul_rn(h, h);
         const float r = fmaf(h, h, -s) + 2.0f * h * l;
-        nh = Sum3::two_sum(nh, s, e);
-        nl += e + r;
+        nh = Sum3::two_sum(nh, s, err);
+        nl += err + r;
     }
     nh = Sum3::two_sum(nh, nl, nl);
-    float rh, rl;
-    rho.pair(rh, rl);
     const float dh = __fmul_rn(rh, rh), dl = fmaf(rh, rh, -dh) + 2.0f * rh * rl;
     qh = __fdiv_rn(nh, dh);
     ql = __fdiv_rn(fmaf(-qh, dl, fmaf(-qh, dh, nh) + nl), dh);
     qh = Sum3::two_sum(qh, ql, ql);
+    return (qh >= 0x1p-90f && qh <= 0x1p100f) || (still && rh >= 0x1p-10f && rh < 4.0f);
 }
 
 // Density and total momentum (half the force included) of a cell in FP64.
@@ -304,6 +316,17 @@ __device__ __forceinline__ void cell_sums(const KParams &p, const S *__restrict_
     T F[3];
     cell_force<L, T>(p, psi, psi_index(p, x, y, z), F);
     for (int a = 0; a < 3; ++a) m[a] = j[a] + 0.5 * (double)F[a];
+}
+
+// |u| of cell s in FP64.
+template <class L, class S>
+__device__ __forceinline__ double cell_speed(const KParams &p, const S *__restrict__ A,
+                                             const typename Store<S>::PsiT *__restrict__ psi, int odd, long long s) {
+    int x, y, z;
+    double rho, m[3];
+    cell_coords(p, s, x, y, z);
+    cell_sums<L, S>(p, A, psi, odd, 2, s, x, y, z, rho, m);
+    return sqrt((m[0] * m[0] + m[1] * m[1] + m[2] * m[2]) / (rho * rho));
 }
 
 // The block's partial from its threads' sums (or maxima).
@@ -372,13 +395,20 @@ __global__ void __launch_bounds__(256) k_reduce(KParams p, const S *__restrict__
 // FP32 arithmetic: density (WHAT 0), momentum (1) and the largest speed (2).  Four blocks per SM: at the
 // 128 registers that it takes uncapped, two, a long chain of additions per cell has too little beside it
 // (the four readouts of 256 x 128 x 128 cells, two / three / four / five blocks: 805 / 719 / 706 / 731 us).
+//
+// Largest speed: pairs of FP32 values rank a thread's cells, and FP64 evaluates the first in rank.  It also
+// evaluates every cell that the pairs cannot rank: one that comes within 2^-36 of the thread's first (the
+// pairs are good to 2^-40), unless its sums are those of the first in every bit (uniform and symmetric
+// flows), and one outside the pairs' range.  So the cell of the largest speed is always among those
+// evaluated, and the result is as accurate as a search in FP64.
 template <class L, class S, int WHAT>
 __global__ void __launch_bounds__(256, 4) k_reduce_f32(KParams p, const S *__restrict__ A, const float *__restrict__ psi,
                                                     int odd, Box box, double *__restrict__ partials) {
     double acc[4] = {0, 0, 0, 0};
     Sum3 sum[3];
-    float bh = -1.0f, bl = 0.0f;               // WHAT 2: the largest speed^2 seen by this thread, its cell
+    float bh = -1.0f, bl = 0.0f;               // WHAT 2: speed^2 of the thread's first cell in rank, the cell
     long long best = -1;
+    __shared__ float first[WHAT == 2 ? 12 : 1][256];                       // its sums
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x; s < p.n; s += stride) {
         int x, y, z;
@@ -407,11 +437,21 @@ __global__ void __launch_bounds__(256, 4) k_reduce_f32(KParams p, const S *__res
 #pragma unroll
                 for (int i = 0; i < L::Q; ++i) rho.add(f[i]);
                 float qh, ql;
-                speed2_pair(rho, sum, L::D, qh, ql);
-                if (qh > bh || (qh == bh && ql > bl)) {
+                const bool ranked = speed2_pair(rho, sum, L::D, qh, ql);
+                const float d = (qh - bh) + (ql - bl), near = 0x1p-36f * bh;
+                const float parts[12] = {rho.h, rho.m, rho.l, sum[0].h, sum[0].m, sum[0].l,
+                                         sum[1].h, sum[1].m, sum[1].l, sum[2].h, sum[2].m, sum[2].l};
+                if (ranked && (best < 0 || d > near)) {
                     bh = qh;
                     bl = ql;
                     best = s;
+#pragma unroll
+                    for (int k = 0; k < 12; ++k) first[k][threadIdx.x] = parts[k];
+                } else if (!(ranked && (d < -near || qh == 0.0f))) {
+                    bool same = ranked;
+#pragma unroll
+                    for (int k = 0; k < 12; ++k) same = same && first[k][threadIdx.x] == parts[k];
+                    if (!same) acc[0] = fmax(acc[0], cell_speed<L, S>(p, A, psi, odd, s));
                 }
             }
         }
@@ -427,13 +467,7 @@ __global__ void __launch_bounds__(256, 4) k_reduce_f32(KParams p, const S *__res
         if ((threadIdx.x & 31) == 0) tops[threadIdx.x >> 5] = top;
         __syncthreads();
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) top = fmaxf(top, tops[w]);
-        if (best >= 0 && bh >= top * (1.0f - 0x1p-20f)) {
-            int x, y, z;
-            double rho, m[3];
-            cell_coords(p, best, x, y, z);
-            cell_sums<L, S>(p, A, psi, odd, WHAT, best, x, y, z, rho, m);
-            acc[0] = fmax(0.0, sqrt((m[0] * m[0] + m[1] * m[1] + m[2] * m[2]) / (rho * rho)));
-        }
+        if (best >= 0 && bh >= top * (1.0f - 0x1p-20f)) acc[0] = fmax(acc[0], cell_speed<L, S>(p, A, psi, odd, best));
     }
     block_partial(acc, WHAT == 2, partials);
 }
