@@ -246,10 +246,9 @@ struct Sum3 {
         m = two_sum(m, e1, e2);
         l = __fadd_rn(l, e2);
     }
-    // (beyond FP32's range the error terms are NaN: the leading part then tells)
-    __device__ __forceinline__ double value() const {
-        return fabsf(h) < INFINITY ? (double)h + ((double)m + (double)l) : (double)h;
-    }
+    // false where the sum has left FP32's range (or a term was not finite): its error terms are then NaN
+    __device__ __forceinline__ bool finite() const { return fabsf(h) < INFINITY; }
+    __device__ __forceinline__ double value() const { return (double)h + ((double)m + (double)l); }
     // the sum as a pair: hi the FP32 value nearest to it
     __device__ __forceinline__ void pair(float &hi, float &lo) const {
         hi = two_sum(h, __fadd_rn(m, l), lo);
@@ -457,8 +456,27 @@ __global__ void __launch_bounds__(256, 4) k_reduce_f32(KParams p, const S *__res
         }
     }
     if constexpr (WHAT < 2) {
+        bool finite = true;
 #pragma unroll
-        for (int a = 0; a < (WHAT ? 3 : 1); ++a) acc[a] = sum[a].value();
+        for (int a = 0; a < (WHAT ? 3 : 1); ++a) {
+            acc[a] = sum[a].value();
+            finite = finite && sum[a].finite();
+        }
+        if (!finite) {
+            // beyond FP32's range: this thread's cells again, in FP64
+            acc[0] = acc[1] = acc[2] = 0.0;
+#pragma unroll 1
+            for (long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x; s < p.n; s += stride) {
+                int x, y, z;
+                cell_coords(p, s, x, y, z);
+                if (!box.holds(x, y, z)) continue;
+                double rho, m[3];
+                cell_sums<L, S>(p, A, psi, odd, WHAT, s, x, y, z, rho, m);
+                if (WHAT == 0) acc[0] += rho;
+                else
+                    for (int a = 0; a < 3; ++a) acc[a] += m[a];
+            }
+        }
     } else {
         // the threads whose cell comes within 2^-20 of the block's largest evaluate it in FP64
         float top = bh;
