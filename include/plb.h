@@ -175,6 +175,10 @@ int plb_init_physical(plb_t *h, const double *rho0, const double *u0);
  * and reported by plb_status / plb_moments / plb_reduce. */
 int plb_step(plb_t *h, int n);
 
+/* How plb_step advanced h since plb_create: counts[0] = launches that took many steps each, counts[1] =
+ * the steps they took (the kernels of a single step took the others).  PLB_EINVAL for NULL arguments. */
+int plb_launch_counts(const plb_t *h, long long counts[2]);
+
 /* Same as plb_step(h, n), with CUDA events recorded on the handle's stream around every
  * launch; ms[0] receives the summed duration of the n psi passes, ms[1] of the n fused
  * force + collide + stream passes (milliseconds).  Synchronises.  For measurement. */
@@ -301,6 +305,10 @@ long long plb_batch_time(const plb_batch_t *b);
  * launched directly (the default stream, a withheld-arrival test launch, or a stream whose
  * capture failed).  PLB_EINVAL for NULL arguments. */
 int plb_batch_launch_counts(const plb_batch_t *b, long long counts[3]);
+
+/* How a batch is split: split[0] = tiles, split[1] = groups of instances stepped one after the other.
+ * PLB_EINVAL for NULL arguments. */
+int plb_batch_split(const plb_batch_t *b, int split[2]);
 
 /* ---------------------------------------------------------------- slab decomposition
  * One D3Q19 lattice of nx x ny x NZ cells, periodic in z, split along z into slabs (one per

@@ -87,6 +87,7 @@ _SIGNATURES = {
     "plb_init_physical": (ctypes.c_int, [_VP, _DP, _DP]),
     "plb_step": (ctypes.c_int, [_VP, ctypes.c_int]),
     "plb_step_timed": (ctypes.c_int, [_VP, ctypes.c_int, _DP]),
+    "plb_launch_counts": (ctypes.c_int, [_VP, ctypes.POINTER(ctypes.c_longlong)]),
     "plb_status": (ctypes.c_int, [_VP]),
     "plb_time": (ctypes.c_longlong, [_VP]),
     "plb_moments": (ctypes.c_int, [_VP, _DP, _DP, _DP]),
@@ -116,6 +117,7 @@ _SIGNATURES = {
     "plb_batch_withhold_arrivals": (ctypes.c_int, [_VP, ctypes.c_uint]),
     "plb_batch_time": (ctypes.c_longlong, [_VP]),
     "plb_batch_launch_counts": (ctypes.c_int, [_VP, ctypes.POINTER(ctypes.c_longlong)]),
+    "plb_batch_split": (ctypes.c_int, [_VP, _IP]),
     "plb_slab_plan": (ctypes.c_int, [ctypes.c_int, _IP, ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_int,
                                      ctypes.POINTER(plb_xfer), ctypes.c_int, _IP]),
     "plb_slab_bind": (ctypes.c_int, [_VP, ctypes.c_int]),
@@ -224,6 +226,12 @@ def plb_step_timed(h, n: int):
     ms = np.zeros(2)
     _check(lib().plb_step_timed(h, int(n), _dptr(ms)))
     return float(ms[0]), float(ms[1])
+
+
+def plb_launch_counts(h) -> dict:
+    c = (ctypes.c_longlong * 2)()
+    _check(lib().plb_launch_counts(h, c))
+    return {"many_step_launches": c[0], "many_steps": c[1]}
 
 
 def plb_status(h):
@@ -353,6 +361,12 @@ def plb_batch_launch_counts(b) -> dict:
     c = (ctypes.c_longlong * 3)()
     _check(lib().plb_batch_launch_counts(b, c))
     return {"graph_captures": c[0], "graph_launches": c[1], "direct_launches": c[2]}
+
+
+def plb_batch_split(b) -> dict:
+    c = (ctypes.c_int * 2)()
+    _check(lib().plb_batch_split(b, c))
+    return {"tiles": c[0], "groups": c[1]}
 
 
 def plb_slab_plan(lattice: int, dims, precision: int, wall_y: int, pass_: int, odd: int) -> list:

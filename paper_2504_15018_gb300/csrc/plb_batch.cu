@@ -499,4 +499,11 @@ int plb_batch_launch_counts(const plb_batch_t *b, long long counts[3]) {
     return PLB_OK;
 }
 
+int plb_batch_split(const plb_batch_t *b, int split[2]) {
+    if (!b || !split) return plb::set_error(PLB_EINVAL, "NULL argument");
+    split[0] = b->ntiles;
+    split[1] = b->ngroups;
+    return PLB_OK;
+}
+
 }  // extern "C"

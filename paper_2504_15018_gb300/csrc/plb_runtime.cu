@@ -550,6 +550,8 @@ int step_tiles(plb_t *h, int n, int coll) {
     }
     if (h->pops2 && (t.nsteps & 1)) std::swap(h->pops, h->pops2);
     h->t += t.nsteps;
+    h->many_launches += 1;
+    h->many_steps += t.nsteps;
     return first + t.nsteps;
 }
 
@@ -581,6 +583,13 @@ int plb_step(plb_t *h, int n) {
         h->t += 1;
     }
     return check_launch();
+}
+
+int plb_launch_counts(const plb_t *h, long long counts[2]) {
+    if (!h || !counts) return fail(PLB_EINVAL, "NULL argument");
+    counts[0] = h->many_launches;
+    counts[1] = h->many_steps;
+    return PLB_OK;
 }
 
 int plb_step_timed(plb_t *h, int n, double ms[2]) {
