@@ -179,6 +179,11 @@ int plb_step(plb_t *h, int n);
  * the steps they took (the kernels of a single step took the others).  PLB_EINVAL for NULL arguments. */
 int plb_launch_counts(const plb_t *h, long long counts[2]);
 
+/* Test hook for failure detection: in the next launch of plb_step that takes many steps, one tile of the
+ * lattice keeps its progress to itself and waits poll at most spin_limit times, so that they run out and
+ * plb_status reports PLB_ETIMEOUT.  Nothing faults or hangs.  0 withdraws it. */
+int plb_withhold_counts(plb_t *h, unsigned spin_limit);
+
 /* Same as plb_step(h, n), with CUDA events recorded on the handle's stream around every
  * launch; ms[0] receives the summed duration of the n psi passes, ms[1] of the n fused
  * force + collide + stream passes (milliseconds).  Synchronises.  For measurement. */
@@ -186,7 +191,8 @@ int plb_step_timed(plb_t *h, int n, double ms[2]);
 
 /* Synchronises the stream and returns PLB_EPSI_DOMAIN / PLB_ENONFINITE if a kernel
  * met such a cell since creation or the last plb_init, PLB_ETIMEOUT if a bounded wait inside
- * a step gave up (the populations are then undefined until the next plb_init), else PLB_OK. */
+ * a step gave up (the populations are then undefined until the next plb_init, plb_set_state or
+ * plb_set_populations, which also clear this error), else PLB_OK. */
 int plb_status(plb_t *h);
 
 /* Number of steps since plb_init; -1 for a NULL handle. */

@@ -87,6 +87,7 @@ _SIGNATURES = {
     "plb_init_physical": (ctypes.c_int, [_VP, _DP, _DP]),
     "plb_step": (ctypes.c_int, [_VP, ctypes.c_int]),
     "plb_step_timed": (ctypes.c_int, [_VP, ctypes.c_int, _DP]),
+    "plb_withhold_counts": (ctypes.c_int, [_VP, ctypes.c_uint]),
     "plb_launch_counts": (ctypes.c_int, [_VP, ctypes.POINTER(ctypes.c_longlong)]),
     "plb_status": (ctypes.c_int, [_VP]),
     "plb_time": (ctypes.c_longlong, [_VP]),
@@ -226,6 +227,10 @@ def plb_step_timed(h, n: int):
     ms = np.zeros(2)
     _check(lib().plb_step_timed(h, int(n), _dptr(ms)))
     return float(ms[0]), float(ms[1])
+
+
+def plb_withhold_counts(h, spin_limit: int):
+    _check(lib().plb_withhold_counts(h, int(spin_limit)))
 
 
 def plb_launch_counts(h) -> dict:

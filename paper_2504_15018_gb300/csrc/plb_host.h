@@ -74,6 +74,7 @@ struct plb_state {
     unsigned *counts;          // step counts of the many-step launch's tiles (NULL: not used)
     plb::TileArgs tiles;       // its split of the lattice, planned at the first step
     int tiles_state;           // 0: not planned yet, 1: planned, -1: not for this lattice
+    unsigned withhold;         // test hook: polling limit of the next many-step launch, whose tile 0 keeps its counts
     long long many_launches;   // many-step launches of plb_step, and the steps they took
     long long many_steps;
     int slab;                  // 1: a z-slab whose first and last planes are ghost planes (plb_slab_*)

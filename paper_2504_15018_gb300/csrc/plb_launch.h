@@ -110,6 +110,7 @@ struct TileArgs {
     int max_own, max_region;  // cells (pairs) of the largest tile, without and with its ring
     int nsteps;
     unsigned spin_limit;
+    int withhold;             // test hook: tile 0 keeps its step counts to itself
 };
 
 struct Launchers {

@@ -139,6 +139,16 @@ cudaError_t clear_counts(plb_t *h) {
     return h->counts ? cudaMemsetAsync(h->counts, 0, plb::kTileWords * sizeof(unsigned), h->stream) : cudaSuccess;
 }
 
+__global__ void k_forget_timeout(unsigned *flags) { atomicAnd(flags, ~(unsigned)plb::FLAG_TIMEOUT); }
+
+// Before the populations are replaced: a wait that gave up is forgotten (the other flags stay).
+cudaError_t forget_timeout(plb_t *h) {
+    if (!h->counts) return cudaSuccess;
+    k_forget_timeout<<<1, 1, 0, h->stream>>>(h->kp.flags);
+    const cudaError_t e = cudaGetLastError();
+    return e != cudaSuccess ? e : clear_counts(h);
+}
+
 int check_launch() {
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(PLB_ECUDA, "kernel launch: %s", cudaGetErrorString(e));
@@ -539,7 +549,9 @@ int step_tiles(plb_t *h, int n, int coll) {
     t.a = h->pops;
     t.b = h->pops2 ? h->pops2 : reinterpret_cast<char *>(h->staging);
     t.counts = h->counts;
-    t.spin_limit = 1u << 22;
+    t.spin_limit = h->withhold ? h->withhold : 1u << 22;
+    t.withhold = h->withhold ? 1 : 0;
+    h->withhold = 0;
     h->kp.salt = (unsigned)h->t;
     cudaError_t e = h->L->tile_run[form](h->kp, coll, t, h->stream);
     if (e != cudaSuccess) {
@@ -583,6 +595,12 @@ int plb_step(plb_t *h, int n) {
         h->t += 1;
     }
     return check_launch();
+}
+
+int plb_withhold_counts(plb_t *h, unsigned spin_limit) {
+    if (!h) return fail(PLB_EINVAL, "NULL handle");
+    h->withhold = spin_limit;
+    return PLB_OK;
 }
 
 int plb_launch_counts(const plb_t *h, long long counts[2]) {
@@ -747,6 +765,7 @@ int plb_set_populations(plb_t *h, const double *f) {
     if (h->view) return fail(PLB_EINVAL, "this lattice belongs to a batch: populations are read-only here");
     const long long n = h->lay.n, chunk = h->lay.chunk;
     double *stg = staging_ptr(h);
+    PLB_CUDA(forget_timeout(h));
     for (long long c0 = 0; c0 < n; c0 += chunk) {
         const long long cn = (n - c0) < chunk ? (n - c0) : chunk;
         for (int i = 0; i < h->lay.Q; ++i)
@@ -787,6 +806,7 @@ int plb_set_state(plb_t *h, const void *host_buf, size_t bytes) {
     if (hdr[0] != (long long)MAGIC || hdr[1] != h->lattice || hdr[2] != h->opts.precision || hdr[3] != h->dims[0] ||
         hdr[4] != h->dims[1] || hdr[5] != h->dims[2])
         return fail(PLB_EINVAL, "state does not match this lattice");
+    PLB_CUDA(forget_timeout(h));
     PLB_CUDA(cudaMemcpyAsync(pops_ptr(h), static_cast<const char *>(host_buf) + 64, plb_state_bytes(h) - 64,
                              cudaMemcpyHostToDevice, h->stream));
     PLB_CUDA(cudaStreamSynchronize(h->stream));

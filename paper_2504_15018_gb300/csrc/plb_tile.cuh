@@ -15,7 +15,8 @@
 // block's stores and read before a fence; populations bypass L1.  The counts only grow, and every
 // launch starts from the block's own count, so nothing has to be cleared between launches.  The
 // launch is cooperative (all tiles resident), and every wait is bounded: one that runs out records
-// FLAG_TIMEOUT and the blocks leave.
+// FLAG_TIMEOUT and the blocks leave, as do those of later launches until the counts are cleared (the
+// tiles stand at different steps, and counts say nothing about neighbours any more).
 //
 // What bounds it: the chain poll -> L2 loads -> psi -> collision -> stores -> release, about 2.7 us a
 // step when every thread has one cell or pair (clock64 of an 8 x 256 lattice: 1300 cycles psi, 930
@@ -115,7 +116,7 @@ __global__ void __maxnreg__((TileThreads<L, S>::regs)) k_tile(KParams p, TileArg
     const unsigned start = *reinterpret_cast<volatile unsigned *>(count);
     S *src = static_cast<S *>(t.a), *dst = static_cast<S *>(t.b);
     for (int s = 0; s < t.nsteps; ++s) {
-        int ok = 1;
+        int ok = s > 0 || ld_relaxed(t.counts) == 0;
         if (s > 0 && watch) {
             unsigned spins = 0;
             while ((int)(ld_relaxed(watch) - (start + (unsigned)s)) < 0) {
@@ -128,7 +129,7 @@ __global__ void __maxnreg__((TileThreads<L, S>::regs)) k_tile(KParams p, TileArg
             }
             fence_acq_rel();
         }
-       if (!__syncthreads_and(ok)) return;
+        if (!__syncthreads_and(ok)) return;
         // ---- psi of the tile and its ring
         Planes<S> A, B;
 #pragma unroll
@@ -203,7 +204,7 @@ __global__ void __maxnreg__((TileThreads<L, S>::regs)) k_tile(KParams p, TileArg
             }
         }
         __syncthreads();
-        if (tid == 0)
+        if (tid == 0 && !(t.withhold && tile == 0))
             asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(count), "r"(start + (unsigned)s + 1) : "memory");
         S *const u = src;
         src = dst;
