@@ -517,54 +517,66 @@ int plb::rebalance_state(plb_state *h) {
 
 namespace {
 
-// Advances a small lattice by as many of n steps as the many-step launch takes (0: none).  In-place lattices borrow the staging area as the second population copy,
-// take an even number of steps (the populations end where they were) and start at even parity.
-int step_tiles(plb_t *h, int n, int coll) {
+// Steps of one launch: a launch holds its SMs to its end, so a longer call is several launches, of about a
+// millisecond each (an FP64 cell costs some eight times an FP32 one), between which the work of other
+// streams gets its turn.  A launch's start (some 10 us) is then a hundredth of it.
+int tile_steps(const plb_t *h) {
+    const long long cells = h->opts.precision == PLB_FP64 ? 1LL << 21 : 1LL << 24;
+    const long long steps = cells / h->lay.n;
+    return steps < 16 ? 16 : (steps > 512 ? 512 : (int)(steps & ~1LL));
+}
+
+// Advances a small lattice by as many of n steps as many-step launches take (taken; 0: none).  In-place
+// lattices borrow the staging area as the second population copy, take an even number of steps (the
+// populations end where they were) and start at even parity.
+int step_tiles(plb_t *h, int n, int coll, int &taken) {
     const int form = h->pops2 ? 1 : 0;
+    taken = 0;
     if (h->tiles_state == 0) {
         const plb::Layout &L = h->lay;
         bool use = h->counts && L.n == L.chunk;        // the staging area holds a second copy
         if (use) use = h->L->tile_plan[form](h->kp, coll, h->tiles);
         h->tiles_state = use ? 1 : -1;
     }
-    if (h->tiles_state < 0) return 0;
-    plb::TileArgs t = h->tiles;
-    int first = 0;
-    if (!h->pops2) {
-        if (h->odd) {
-            // one in-place step brings the natural layout back
-            if (n < 3) return 0;
-            h->kp.salt = (unsigned)h->t;
-            h->L->psi(h->kp, h->pops, h->psi, 1, h->stream);
-            h->L->collide[coll](h->kp, h->pops, h->psi, 1, h->stream);
-            h->odd = 0;
-            h->t += 1;
-            first = 1;
+    if (h->tiles_state < 0) return PLB_OK;
+    if (!h->pops2 && h->odd) {
+        // one in-place step brings the natural layout back
+        if (n < 3) return PLB_OK;
+        h->kp.salt = (unsigned)h->t;
+        h->L->psi(h->kp, h->pops, h->psi, 1, h->stream);
+        h->L->collide[coll](h->kp, h->pops, h->psi, 1, h->stream);
+        h->odd = 0;
+        h->t += 1;
+        taken = 1;
+        const int st = check_launch();                 // (before the error of a launch of tiles is dropped)
+        if (st != PLB_OK) return st;
+    }
+    const int most = tile_steps(h);
+    while (n - taken >= 2) {
+        plb::TileArgs t = h->tiles;
+        t.nsteps = n - taken < most ? n - taken : most;
+        if (!h->pops2) t.nsteps &= ~1;
+        t.a = h->pops;
+        t.b = h->pops2 ? h->pops2 : reinterpret_cast<char *>(h->staging);
+        t.counts = h->counts;
+        t.spin_limit = h->withhold ? h->withhold : 1u << 22;
+        t.withhold = h->withhold ? 1 : 0;
+        h->withhold = 0;
+        h->kp.salt = (unsigned)h->t;
+        cudaError_t e = h->L->tile_run[form](h->kp, coll, t, h->stream);
+        if (e != cudaSuccess) {
+            // the tiles do not fit this context (fewer SMs than the device reports): the other kernels do
+            cudaGetLastError();
+            h->tiles_state = -1;
+            return PLB_OK;
         }
-        t.nsteps = (n - first) & ~1;
-    } else {
-        t.nsteps = n;
+        if (h->pops2 && (t.nsteps & 1)) std::swap(h->pops, h->pops2);
+        h->t += t.nsteps;
+        h->many_launches += 1;
+        h->many_steps += t.nsteps;
+        taken += t.nsteps;
     }
-    if (t.nsteps < 2) return first;
-    t.a = h->pops;
-    t.b = h->pops2 ? h->pops2 : reinterpret_cast<char *>(h->staging);
-    t.counts = h->counts;
-    t.spin_limit = h->withhold ? h->withhold : 1u << 22;
-    t.withhold = h->withhold ? 1 : 0;
-    h->withhold = 0;
-    h->kp.salt = (unsigned)h->t;
-    cudaError_t e = h->L->tile_run[form](h->kp, coll, t, h->stream);
-    if (e != cudaSuccess) {
-        // the tiles do not fit this context (fewer SMs than the device reports): the other kernels do
-        cudaGetLastError();
-        h->tiles_state = -1;
-        return first;
-    }
-    if (h->pops2 && (t.nsteps & 1)) std::swap(h->pops, h->pops2);
-    h->t += t.nsteps;
-    h->many_launches += 1;
-    h->many_steps += t.nsteps;
-    return first + t.nsteps;
+    return PLB_OK;
 }
 
 }  // namespace
@@ -576,7 +588,10 @@ int plb_step(plb_t *h, int n) {
     if (h->view) return fail(PLB_EINVAL, "this lattice belongs to a batch: use plb_batch_step");
     if (h->slab) return fail(PLB_EINVAL, "this lattice is a slab: step it with plb_slab_pass and plb_slab_exchange");
     const int coll = h->opts.collision == PLB_MRT ? 1 : 0;
-    n -= step_tiles(h, n, coll);
+    int taken = 0;
+    const int st = step_tiles(h, n, coll, taken);
+    if (st != PLB_OK) return st;
+    n -= taken;
     if (h->pops2) {
         // single pass: read the current copy, push into the other, swap
         for (int k = 0; k < n; ++k) {
