@@ -286,8 +286,8 @@ int plb_batch_status(plb_batch_t *b);
 /* Clears a recorded barrier timeout. */
 int plb_batch_reset_error(plb_batch_t *b);
 
-/* Tile size in cells (no less than a row or 256 threads' cells), resident 256-thread
- * blocks per SM, and the barrier's polling limit (0 keeps the default, about a second or more).
+/* Tile size in cells at two cells per thread (tile_cells / 2 cells where a thread has one: FP64, odd nx;
+ * no less than a row or 256 threads' cells; 512 is the default), resident 256-thread blocks per SM, and the barrier's polling limit (0 keeps the default, about a second or more).
  * A non-positive tile_cells or blocks_per_sm keeps the current value. */
 int plb_batch_configure(plb_batch_t *b, int tile_cells, int blocks_per_sm, unsigned spin_limit);
 

@@ -26,6 +26,7 @@ namespace {
 size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
 
 constexpr unsigned kDefaultSpinLimit = 1u << 22;   // ~ 1-4 s of polling
+constexpr int kDefaultTileCells = 512;             // one unit per thread of a block
 constexpr double kGroupBytes = 72e6;               // working set of a launch that stays in L2 (129 MB)
 
 struct InstLayout {
@@ -97,7 +98,7 @@ struct plb_batch_state {
     cudaStream_t stream;
     const plb::Launchers *L;
     int nsm;
-    int tile_cells;        // cells per tile (0: one unit per thread)
+    int tile_cells;        // cells per tile, at two cells per thread
     int blocks_per_sm;     // resident blocks requested per SM
     int max_blocks_per_sm; // occupancy limit of the kernel
     int ntiles;
@@ -115,14 +116,14 @@ struct plb_batch_state {
 namespace {
 
 int build_tiles(plb_batch_t *b) {
-    // Tiles of tile_cells cells (by default of one unit per thread) in instance order; a block takes
-    // consecutive ones.  Whole rows per tile, dealt out in turn, left threads idle and the fullest block
+    // Tiles of tile_cells / 2 units (a thread's work: two cells, or one in FP64 and for odd nx; by default
+    // one unit per thread of a block) in instance order; a block takes consecutive ones.  Whole rows per tile, dealt out in turn, left threads idle and the fullest block
     // with 16 rounds where 13.2 would do (60 lattices of 64^2 .. 512^2).
     std::vector<plb::BatchTile> tiles;
     for (int k = 0; k < b->n; ++k) {
         const plb::BatchInst &in = b->host_insts[k];
         const int ny = b->views[k]->dims[1], nz = b->views[k]->dims[2], units = in.upr * ny;
-        int per = b->tile_cells > 0 ? b->tile_cells / (in.pair ? 2 : 1) : 256;
+        int per = b->tile_cells / 2;
         // no finer than a row (or a block's threads): the tile table's size
         const int least = in.upr < 256 ? in.upr : 256;
         if (per < least) per = least;
@@ -254,7 +255,7 @@ int plb_batch_create(int lattice, int n, const plb_instance *inst, void *dev_wor
     if (occ < 1) return fail_destroy(plb::set_error(PLB_EUNSUPPORTED, "batch kernel does not fit on an SM"));
     b->max_blocks_per_sm = occ;
     b->blocks_per_sm = occ;
-    b->tile_cells = 0;
+    b->tile_cells = kDefaultTileCells;
     b->views.resize(n, nullptr);
     b->host_insts.resize(n);
     for (int k = 0; k < n; ++k) {
@@ -451,7 +452,7 @@ int plb_batch_withhold_arrivals(plb_batch_t *b, unsigned count) {
 
 int plb_batch_autotune(plb_batch_t *b, int steps_per_candidate, int *tile_cells, int *blocks_per_sm, double *best_ms) {
     if (!b || steps_per_candidate < 1) return plb::set_error(PLB_EINVAL, "bad argument");
-    const int cand_tiles[] = {512, 1024, 2048, 4096, 8192, 16384};
+    const int cand_tiles[] = {kDefaultTileCells, 1024, 2048, 4096, 8192, 16384};
     float best = 1e30f;
     int bt = b->tile_cells, bb = b->blocks_per_sm;
     cudaEvent_t e0, e1;
