@@ -78,7 +78,7 @@ bool arena_layout(int lattice, int n, const plb_instance *d, ArenaLayout &A) {
     A.off_partials = off;
     off = align256(off + (size_t)1024 * 4 * sizeof(double));
     A.off_out = off;
-    off = align256(off + 4 * sizeof(double));
+    off = align256(off + plb::kReduceOut * sizeof(double));
     A.off_staging = off;
     const int per_cell = A.Q > A.inst[0].lay.D + 2 ? A.Q : A.inst[0].lay.D + 2;
     off = align256(off + (size_t)A.chunk * per_cell * sizeof(double));

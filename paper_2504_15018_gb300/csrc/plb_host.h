@@ -17,6 +17,9 @@ int solve_coexistence(const plb_eos_params &e, double &rho_v, double &rho_l, dou
 bool needs_coexistence(double tau, const plb_opts &o);
 int si_convert(const double si[6], const double lat[3], double xi, double out[11]);
 
+// Values of a reduction's result: four sums or maxima, and the error flags.
+constexpr int kReduceOut = 5;
+
 // Byte layout of the caller's device workspace (every region 256-byte aligned).
 struct Layout {
     int Q, D;
@@ -65,7 +68,7 @@ struct plb_state {
     char *ws;
     char *pops, *psi;          // population store (the current copy), padded psi field
     char *pops2;               // PLB_STREAM_FUSED: the copy the next step writes (else NULL)
-    double *partials, *out;    // reduction partials (lay.max_blocks x 4), final values (4)
+    double *partials, *out;    // reduction partials (lay.max_blocks x 4), final values (kReduceOut)
     double *staging;           // host<->device staging (lay.chunk cells)
     cudaStream_t stream;
     long long t;

@@ -80,7 +80,7 @@ bool make_layout(int lattice, const int dims[3], int precision, Layout &L, int s
     L.off_partials = off;
     off = align256(off + (size_t)L.max_blocks * 4 * sizeof(double));
     L.off_out = off;
-    off = align256(off + 5 * sizeof(double));
+    off = align256(off + kReduceOut * sizeof(double));
     L.off_staging = off;
     const int per_cell = L.Q > L.D + 2 ? L.Q : L.D + 2;
     // (a small lattice's staging area also serves as the second population copy of many-step launches)
@@ -745,7 +745,7 @@ int plb_reduce(plb_t *h, int what, const int lo[3], const int hi[3], double *out
     reduce_final_launch(partials, nblocks, what == PLB_UMAX, h->kp.flags, dout, h->stream);
     st = check_launch();
     if (st) return st;
-    double res[5];                 // four sums or maxima, the error flags
+    double res[plb::kReduceOut];
     PLB_CUDA(cudaMemcpyAsync(res, dout, sizeof(res), cudaMemcpyDeviceToHost, h->stream));
     PLB_CUDA(cudaStreamSynchronize(h->stream));
     switch (what) {
