@@ -154,7 +154,9 @@ __device__ __forceinline__ double quotient(double a, double b, const Recip &r) {
     const bool zero = (hi << 1 | (unsigned)__double2loint(a)) == 0u;
     if (((hi >> 20 & 0x7ffu) - 123u >= 1800u && !zero) || er - 923u >= 200u) return a / b;
     const double q = __fma_rn(a, r.h, __dmul_rn(a, r.l));
-    return __fma_rn(__fma_rn(-b, q, a), r.h, q);
+    const double v = __fma_rn(__fma_rn(-b, q, a), r.h, q);
+    // (a zero dividend: the sums above can lose the sign of the quotient)
+    return zero ? __hiloint2double((int)((hi ^ (unsigned)__double2hiint(b)) & 0x80000000u), 0) : v;
 }
 
 // 1 / b as a pair of doubles.
