@@ -239,9 +239,10 @@ __device__ __forceinline__ double fdiv(double a, double b) { return a / b; }
 // ----------------------------------------------------------------- utilities
 // Start of a step kernel: the next kernel of the stream may begin to launch (its blocks wait in turn),
 // then wait for the kernel before this one.  Launches of step kernels carry the matching attribute
-// (Launch::go), so that launch latency and the ramp of a grid run under the tail of the one before it.
-// Microseconds a step, before and after: 64^3 FP32 18.5 and 14.0, 127 x 95 x 63 FP32 33.6 and 29.8, 160^3
-// FP16 with stochastic rounding 136 and 131; the single pass (750 us a kernel) gained nothing and goes without.
+// (Launch::go; Launch::go_long where the grid is small and its blocks long), so that launch latency and the
+// ramp of a grid run under the tail of the one before it.  Microseconds a step, before and after: 64^3 FP32
+// 18.5 and 14.0, 127 x 95 x 63 FP32 33.6 and 29.8, 160^3 FP16 with stochastic rounding 136 and 131; the single
+// pass (750 us a kernel) gained nothing and goes without.
 __device__ __forceinline__ void step_kernel_begin() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");

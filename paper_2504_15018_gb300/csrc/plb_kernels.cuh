@@ -4,6 +4,9 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <map>
+#include <utility>
+
 #include "plb_device.cuh"
 #include "plb_launch.h"
 #include "plb_batch.cuh"
@@ -559,16 +562,35 @@ template <class L, class S> struct Launch {
     // (step_kernel_begin waits for that one).
     template <class... P, class... Args>
     static void go(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, const Args &...args) {
+        go_if(true, kernel, grid, block, st, args...);
+    }
+    template <class... P, class... Args>
+    static void go_if(bool early, void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, const Args &...args) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = grid;
         cfg.blockDim = block;
         cfg.stream = st;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        attr[0].val.programmaticStreamSerializationAllowed = early ? 1 : 0;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+    }
+    // The same for the collision kernels whose blocks run long (FP64, and FP16 D3Q19): early only if the grid
+    // fills every SM.  Blocks that come early pile up on the SMs that come free first, and the fullest SM then
+    // ends the step.  Microseconds a step, one step a call, always early and now: FP64 24^3 99 and 45, 32^3 104
+    // and 74, 200^2 84 and 51; FP16 64^3 26 and 17, with a wait after each step 41 and 27.
+    template <class... P, class... Args>
+    static void go_long(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, const Args &...args) {
+        static thread_local std::map<std::pair<const void *, unsigned>, int> cache;
+        const unsigned threads = block.x * block.y;
+        int &resident = cache[{(const void *)kernel, threads}];
+        if (resident == 0 &&
+            (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, kernel, (int)threads, 0) != cudaSuccess ||
+             resident < 1))
+            resident = 1;
+        go_if((long long)grid.x * grid.y * grid.z >= (long long)resident * sm_count(), kernel, grid, block, st, args...);
     }
     static Planes<S> planes(const KParams &p, const void *A) {
         Planes<S> pl;
@@ -641,12 +663,12 @@ template <class L, class S> struct Launch {
         const dim3 grid(sp.segments, (p.ny + sp.rows - 1) / sp.rows, (p.nzl + PLB_STAGED_ZC - 1) / PLB_STAGED_ZC);
         if constexpr (Store<S>::SHIFT) {
             if (p.stochastic) {
-                go(k_collide_staged<L, S, MRT, ODD, true, WIDE>, grid, sp.threads, st, p, planes(p, A),
+                go_long(k_collide_staged<L, S, MRT, ODD, true, WIDE>, grid, sp.threads, st, p, planes(p, A),
                    (const float *)psi, sp);
                 return;
             }
         }
-        go(k_collide_staged<L, S, MRT, ODD, false, WIDE>, grid, sp.threads, st, p, planes(p, A), (const float *)psi, sp);
+        go_long(k_collide_staged<L, S, MRT, ODD, false, WIDE>, grid, sp.threads, st, p, planes(p, A), (const float *)psi, sp);
     }
     template <int MRT, bool ODD> static void collide_t(const KParams &p, void *A, const void *psi, cudaStream_t st) {
         dim3 grid, block;
@@ -686,9 +708,9 @@ template <class L, class S> struct Launch {
         if constexpr (std::is_same<S, double>::value) {
             dims3(p, grid, block, 128);
             if (p.n < (1LL << 31))
-                go(k_collide_plain<L, MRT, ODD, int>, grid, block, st, p, planes(p, A), (const double *)psi);
+                go_long(k_collide_plain<L, MRT, ODD, int>, grid, block, st, p, planes(p, A), (const double *)psi);
             else
-                go(k_collide_plain<L, MRT, ODD, long long>, grid, block, st, p, planes(p, A), (const double *)psi);
+                go_long(k_collide_plain<L, MRT, ODD, long long>, grid, block, st, p, planes(p, A), (const double *)psi);
             return;
         }
         dims3(p, grid, block);
