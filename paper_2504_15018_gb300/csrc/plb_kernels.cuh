@@ -676,7 +676,8 @@ template <class L, class S> struct Launch {
             if constexpr (std::is_same<L, D3Q19>::value) {
                 if (use_pair(p) && (std::is_same<S, __half>::value ? PLB_STAGED_HALF : PLB_STAGED_FLOAT) != 0) {
                     bool wide = false;
-                    const StagedSplit sp = staged_split(p.nx / 2, p.ny, wide);
+                    const StagedSplit sp = staged_split(p.nx / 2, p.ny, (p.nzl + PLB_STAGED_ZC - 1) / PLB_STAGED_ZC,
+                                                        sm_count(), wide);
                     if (wide) staged_run<MRT, ODD, true>(p, A, psi, sp, st);
                     else staged_run<MRT, ODD, false>(p, A, psi, sp, st);
                     return;

@@ -76,13 +76,21 @@ struct StagedSplit {
     int width, rows, segments, threads;
 };
 
-// The split with the fewest threads, counting idle ones.  64 pairs of one row unless the wide shape
-// needs a tenth less (a row of 80 pairs took one full and one quarter-full block: now two rows are one
-// block of 160).  At least 128 threads, since the wide shape's shared memory allows eight blocks per SM,
-// and whole rows or 128-byte segments.  Step of 160^3 cells with stochastic rounding: 176 -> 136 us.
-inline StagedSplit staged_split(int pairs, int ny, bool &wide) {
+// The split with the least work on the fullest SM: its share of the blocks, times their threads, idle ones
+// counted.  64 pairs of one row unless the wide shape needs a fifth less (a row of 80 pairs took one full and
+// one quarter-full block: now two rows are one block of 160; but the wide blocks of a small lattice are few,
+// and leave SMs idle or unevenly filled).  At least 128 threads, since the wide shape's shared memory allows
+// eight blocks per SM, and whole rows or 128-byte segments.
+// Microseconds a step, one step a call, fewest threads in all and now: FP16 24^3 20 and 15, 80^3 29 and 22,
+// 96^3 34 and 31, with stochastic rounding 184 x 47 x 81 43 and 38, 72^3 35 and 30; 160^3 109 and 109 (139 with
+// plain blocks).
+inline StagedSplit staged_split(int pairs, int ny, int chunks, int sms, bool &wide) {
+    auto fullest = [&](int threads, int segments, int rows) {
+        const long long blocks = (long long)segments * ((ny + rows - 1) / rows) * chunks;
+        return (double)((blocks + sms - 1) / sms) * threads;
+    };
     StagedSplit best = {64, 1, (pairs + 63) / 64, 64};
-    double least = 0.9 * 64.0 * best.segments * ny;
+    double least = 0.8 * fullest(64, best.segments, 1);
     wide = false;
     for (int segments = 1; segments <= (pairs + 9) / 10 && segments <= 64; ++segments) {
         const int width = (pairs + segments - 1) / segments;
@@ -91,9 +99,9 @@ inline StagedSplit staged_split(int pairs, int ny, bool &wide) {
         for (int rows = 1; rows <= ny && rows * width <= StagedShape<true>::THREADS; ++rows) {
             if (rows * (width + 2) > StagedShape<true>::WORDS) break;
             const int threads = (rows * width + 31) / 32 * 32;
-            const double all = (double)threads * segments * ((ny + rows - 1) / rows);
-            if (threads >= 128 && all < least) {
-                least = all;
+            const double most = fullest(threads, segments, rows);
+            if (threads >= 128 && most < least) {
+                least = most;
                 best = {width, rows, segments, threads};
                 wide = true;
             }
