@@ -578,9 +578,10 @@ template <class L, class S> struct Launch {
         cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
     }
     // The same for the collision kernels whose blocks run long (FP64, and FP16 D3Q19): early only if the grid
-    // fills every SM.  Blocks that come early pile up on the SMs that come free first, and the fullest SM then
-    // ends the step.  Microseconds a step, one step a call, always early and now: FP64 24^3 99 and 45, 32^3 104
-    // and 74, 200^2 84 and 51; FP16 64^3 26 and 17, with a wait after each step 41 and 27.
+    // fills every SM or leaves half of them free.  Blocks that come early pile up on the SMs that come free
+    // first, and the fullest SM then ends the step.  Microseconds a step, one step a call, early and not: FP64
+    // 24^3 (144 blocks) 99 and 45, 32^3 104 and 74, 200^2 84 and 51, 16^2 (4 blocks) 21 and 23; FP16 64^3 26 and
+    // 17, with a wait after each step 41 and 27, 10 x 16 x 9 (32 blocks) 13 and 15, 160^3 108 and 111.
     template <class... P, class... Args>
     static void go_long(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, const Args &...args) {
         static thread_local std::map<std::pair<const void *, unsigned>, int> cache;
@@ -590,7 +591,8 @@ template <class L, class S> struct Launch {
             (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, kernel, (int)threads, 0) != cudaSuccess ||
              resident < 1))
             resident = 1;
-        go_if((long long)grid.x * grid.y * grid.z >= (long long)resident * sm_count(), kernel, grid, block, st, args...);
+        const long long n = (long long)grid.x * grid.y * grid.z;
+        go_if(n >= (long long)resident * sm_count() || n <= sm_count() / 2, kernel, grid, block, st, args...);
     }
     static Planes<S> planes(const KParams &p, const void *A) {
         Planes<S> pl;
