@@ -861,14 +861,29 @@ template <class L, class S> struct Launch {
     }
     // Splits the lattice into tiles: the split with the least cost, which is the work of the fullest SM
     // (throughput) plus 256 threads' worth for every pass of a block over its cells (latency).
-    // Which lattices: up to 2^18 cells (the staging area then holds the second copy; at 64^3 FP32 the
-    // tiles still win, 10.8 us a step against 14.6), FP64 D3Q19 only to 2^14 (bound by the FP64 pipe, where
-    // the ring's psi is extra work: 24^3 41 us against 47, 32^3 126 against 123).
+    // Which lattices and calls: those whose steps are then faster than by the kernels of a single step, of up to
+    // 2^18 cells (the staging area holds the second copy).  A launch of tiles costs about 5 us more than its
+    // steps, so larger lattices want more steps a call.  Microseconds a step, tiles and single steps:
+    //   FP32 D3Q19, two cells a thread, 10 steps a call: 44^3 6.9 and 8.3, 48^3 7.3 and 8.4, 50^3 8.5 and 8.6, 60^3
+    //     10.6 and 10.3, 100 steps: 50^3 8.0 and 8.6, 60^3 10.1 and 10.3, 64^3 11.0 and 10.7; one cell, 10 steps:
+    //     33 x 32^2 5.2 and 6.8, 41 x 40^2 6.8 and 7.4, 49 x 48^2 8.6 and 8.5 (100 steps 8.1 and 8.4), 61 x 60^2
+    //     12.8 and 10.7
+    //   FP16 D3Q19: 64^3 10.7 and 17.5; one cell: 49 x 48^2 8.3 and 8.9, 63^3 13.6 and 11.5
+    //   FP64 D2Q9: 256^2 61 and 70, 362^2 124 and 129, 400^2 152 and 156, 512^2 223 and 213; FP64 D3Q19 is bound
+    //     by the FP64 pipe, where the ring's psi is extra work
+    //   FP32 D2Q9 with 2 / 4 / 6 / 10 steps a call: 256^2 5.2 / 4.7 / 4.2 / 3.9 and 5.2, 362^2 6.3 / 5.2 / 4.9 / 4.6
+    //     and 5.8, 512^2 8.3 / 7.3 / 6.9 / 6.6 and 7.1, one cell, 511^2 9.3 / 8.1 / 7.6 / 7.2 and 7.2
     template <int FORM> static bool tile_plan(const KParams &p, int mrt, TileArgs &t) {
         const void *k = tile_kernel<FORM>(p, mrt);
         const int w = !std::is_same<S, double>::value && p.nx % 2 == 0 ? 2 : 1;
         const int nw = p.nx / w, sms = sm_count();
-        if (p.n > (std::is_same<S, double>::value && L::D == 3 ? 1LL << 14 : 1LL << 18)) return false;
+        constexpr bool d3 = L::D == 3, fp64 = std::is_same<S, double>::value, fp32 = std::is_same<S, float>::value;
+        const long long most_cells = fp64 ? (d3 ? 1 << 14 : 10 << 14)
+                                   : FORM || !d3 ? 1 << 18 : fp32 ? (w == 2 ? 14 << 14 : 7 << 14) : (w == 2 ? 1 << 18 : 1 << 17);
+        if (p.n > most_cells) return false;
+        const long long work = p.n * (2 / w);
+        t.least = FORM || fp64 || (d3 && !fp32 && w == 2) || work <= 1 << 16 ? 2
+                : d3 && fp32 && w == 2 && p.n > 7 << 14 ? 16 : work <= 13 << 14 ? 4 : work <= 1 << 18 ? 6 : 10;
         const size_t most = 200 * 1024;
         if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) != cudaSuccess) {
             cudaGetLastError();

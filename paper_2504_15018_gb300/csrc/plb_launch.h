@@ -108,6 +108,7 @@ struct TileArgs {
     int gx, gy, gz;
     int threads;              // per block
     int max_own, max_region;  // cells (pairs) of the largest tile, without and with its ring
+    int least;                // steps below which the kernels of a single step are faster
     int nsteps;
     unsigned spin_limit;
     int withhold;             // test hook: tile 0 keeps its step counts to itself

@@ -541,7 +541,7 @@ int step_tiles(plb_t *h, int n, int coll, int &taken) {
     if (h->tiles_state < 0) return PLB_OK;
     if (!h->pops2 && h->odd) {
         // one in-place step brings the natural layout back
-        if (n < 3) return PLB_OK;
+        if (n < h->tiles.least + 1) return PLB_OK;
         h->kp.salt = (unsigned)h->t;
         h->L->psi(h->kp, h->pops, h->psi, 1, h->stream);
         h->L->collide[coll](h->kp, h->pops, h->psi, 1, h->stream);
@@ -552,7 +552,7 @@ int step_tiles(plb_t *h, int n, int coll, int &taken) {
         if (st != PLB_OK) return st;
     }
     const int most = tile_steps(h);
-    while (n - taken >= 2) {
+    while (n - taken >= h->tiles.least) {
         plb::TileArgs t = h->tiles;
         t.nsteps = n - taken < most ? n - taken : most;
         if (!h->pops2) t.nsteps &= ~1;
