@@ -168,11 +168,12 @@ int plb_init(plb_t *h, const double *rho0, const double *u0);
  * domain is reported by plb_status. */
 int plb_init_physical(plb_t *h, const double *rho0, const double *u0);
 
-/* Advances n time steps (two kernels per step: psi pass, then the fused force +
- * collide + stream pass; lattices of up to 2^18 cells take many steps in one launch, with
- * the same result).  Asynchronous; returns launch errors only.  Device-side
- * faults of the method (psi domain, non-finite density) are recorded in a device flag
- * and reported by plb_status / plb_moments / plb_reduce. */
+/* Advances n time steps: two kernels per step (psi pass, then the fused force + collide + stream
+ * pass), or one (PLB_STREAM_FUSED).  Where that is faster, a small lattice (up to 2^18 cells, fewer
+ * for some storages and widths) takes many steps in one launch, in calls of at least 2 to 16 steps by
+ * its size, with the same result; plb_launch_counts tells.  Asynchronous; returns launch errors
+ * only.  Device-side faults of the method (psi domain, non-finite density) are recorded in a device
+ * flag and reported by plb_status / plb_moments / plb_reduce. */
 int plb_step(plb_t *h, int n);
 
 /* How plb_step advanced h since plb_create: counts[0] = launches that took many steps each, counts[1] =
@@ -184,8 +185,8 @@ int plb_launch_counts(const plb_t *h, long long counts[2]);
  * plb_status reports PLB_ETIMEOUT.  Nothing faults or hangs.  0 withdraws it. */
 int plb_withhold_counts(plb_t *h, unsigned spin_limit);
 
-/* Same as plb_step(h, n), with CUDA events recorded on the handle's stream around every
- * launch; ms[0] receives the summed duration of the n psi passes, ms[1] of the n fused
+/* Advances n time steps as plb_step does, by the kernels of a single step for every lattice (the
+ * same result), with CUDA events recorded on the handle's stream around every launch; ms[0] receives the summed duration of the n psi passes, ms[1] of the n fused
  * force + collide + stream passes (milliseconds).  Synchronises.  For measurement. */
 int plb_step_timed(plb_t *h, int n, double ms[2]);
 
@@ -204,8 +205,8 @@ long long plb_time(const plb_t *h);
  * PLB_EPSI_DOMAIN / PLB_ENONFINITE (as plb_status), PLB_ECUDA. */
 int plb_moments(plb_t *h, double *rho, double *u, double *p);
 
-/* A reduction over the box lo <= (x, y, z) < hi (clipped to the lattice; NULL = whole), summed in
- * FP64 in a fixed order (deterministic).  out receives 1 value (3 for PLB_MOMENTUM).
+/* A reduction over the box lo <= (x, y, z) < hi (clipped to the lattice; NULL = whole), summed in a
+ * fixed order (deterministic) with at least FP64's precision.  out receives 1 value (3 for PLB_MOMENTUM).
  * Synchronises.  Errors: PLB_EINVAL (NULL handle or out, unknown reduction, empty box),
  * PLB_EPSI_DOMAIN / PLB_ENONFINITE (as plb_status), PLB_ECUDA. */
 int plb_reduce(plb_t *h, int what, const int lo[3], const int hi[3], double *out);
@@ -293,7 +294,7 @@ int plb_batch_configure(plb_batch_t *b, int tile_cells, int blocks_per_sm, unsig
 
 /* Times steps_per_candidate steps for every tile size in {512, ..., 16384} cells and every
  * resident count from 1 block per SM to the kernel's occupancy limit (at most 4; the kernel
- * is compiled for 3 D2Q9 / 2 D3Q19 blocks per SM without spilling), keeps the fastest, and reports it (any output may be NULL; best_ms is per
+ * is compiled for 3 D2Q9 / 2 D3Q19 blocks per SM), keeps the fastest, and reports it (any output may be NULL; best_ms is per
  * step).  The timed steps advance the batch. */
 int plb_batch_autotune(plb_batch_t *b, int steps_per_candidate, int *tile_cells, int *blocks_per_sm, double *best_ms);
 

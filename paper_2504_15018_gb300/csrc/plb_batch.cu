@@ -25,9 +25,14 @@ namespace {
 
 size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
 
-constexpr unsigned kDefaultSpinLimit = 1u << 22;   // ~ 1-4 s of polling
+constexpr unsigned kDefaultSpinLimit = 1u << 22;   // about 1.6 s of polling
 constexpr int kDefaultTileCells = 512;             // one unit per thread of a block
-constexpr double kGroupBytes = 72e6;               // working set of a launch that stays in L2 (129 MB)
+// Working set of a group that stays in L2 (129 MB), with room for what streams through.  Microseconds a step with
+// groups and without, 20 steps a call: D2Q9 FP32 batches of 110 MB and less are one group either way, 133 MB
+// 65.5 and 67.2, 146 MB 66.4 and 71.4, 186 MB (MRT) 94 and 102, 252 MB 130 and 133; D3Q19 FP32 377 MB 188 and 197,
+// FP16 219 MB 199 and 196.  A call of two steps reuses little and pays for the groups' barriers: 133 MB 71.9 and
+// 70.0, 252 MB 143 and 136.
+constexpr double kGroupBytes = 72e6;
 
 struct InstLayout {
     plb::Layout lay;

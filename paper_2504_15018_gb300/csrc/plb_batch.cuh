@@ -9,8 +9,10 @@
 
 namespace plb {
 
-// Minimum resident 256-thread blocks per SM requested from the register allocator: the
-// most that fit without spilling (D2Q9: 80 registers, 3 blocks; D3Q19 MRT: 128, 2 blocks).
+// Minimum resident 256-thread blocks per SM requested from the register allocator (D2Q9: 80 registers, 3
+// blocks; D3Q19: 128, 2 blocks).  Most kernels spill a little there (24 to 72 bytes; D3Q19 FP64 BGK 256), which
+// costs less than a block fewer: 24 D3Q19 lattices of 24 to 64 a side, FP32 BGK / MRT 81 / 84 us a step (107 / 114
+// before the even tiles, with 0 / 12 bytes), eight in FP64 1235 / 2012 (2533 / 4013).
 template <class L> struct BatchMinBlocks { static constexpr int value = L::Q == 9 ? 3 : 2; };
 
 // Grid-wide barrier with a bounded wait.  Returns false (in every thread of the block) when

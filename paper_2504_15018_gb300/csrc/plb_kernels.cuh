@@ -232,7 +232,7 @@ __global__ void k_set_pops(KParams p, S *__restrict__ A, const double *__restric
 // population in FP64 took about 100 of them per cell, ten times the HBM time.  FP32 storage adds with
 // error-free transformations on the FP32 pipe instead and converts once per thread; the speed
 // maximum is searched in pairs of FP32 values, and FP64 evaluates the candidates only.  Mass, momentum,
-// maximum speed and moments of 256 x 128 x 128 cells, D3Q19 FP32: 2140 -> 706 us.
+// maximum speed and moments of 256 x 128 x 128 cells, D3Q19 FP32: 2140 -> 713 us.
 
 // A sum of FP32 values in three FP32 parts, each the rounding error of the one before (TwoSum, Knuth
 // 1969; the cascade of Ogita, Rump and Oishi 2005): about 70 bits, where FP64 keeps 53.
@@ -786,10 +786,9 @@ template <class L, class S> struct Launch {
         }
         return nb;
     }
-    // single pass: tiles of 64 x 16 (FP32) or 64 x 32 (FP16) cells, each block walking a chunk
-    // of zc planes.  The chunk
-    // count minimises (waves of resident blocks) x (planes per chunk + 0.5): a block also forms
-    // psi of the two planes before its chunk, at about a third of a collided plane's cost each,
+    // single pass: tiles of FusedTile's size, each block walking a chunk of zc planes.  The chunk count minimises (waves of resident blocks) x (planes per chunk + 0.5): a block also forms
+    // psi of the two planes before its chunk, at about a third of a collided plane's cost each
+    // (measured with tiles of 64 x 16 and kept for 64 x 8),
     // and the last wave of a grid that is not a multiple of the resident blocks runs partly idle.
     template <int MRT> static void fused_t(const KParams &p, const void *A, void *B, cudaStream_t st) {
         if constexpr (!std::is_same<S, double>::value) {

@@ -559,7 +559,7 @@ int step_tiles(plb_t *h, int n, int coll, int &taken) {
         t.a = h->pops;
         t.b = h->pops2 ? h->pops2 : reinterpret_cast<char *>(h->staging);
         t.counts = h->counts;
-        t.spin_limit = h->withhold ? h->withhold : 1u << 22;
+        t.spin_limit = h->withhold ? h->withhold : 1u << 22;       // about 0.7 s of polling
         t.withhold = h->withhold ? 1 : 0;
         h->withhold = 0;
         h->kp.salt = (unsigned)h->t;

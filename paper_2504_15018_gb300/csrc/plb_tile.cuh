@@ -21,9 +21,9 @@
 // What bounds it: the chain poll -> L2 loads -> psi -> collision -> stores -> release, about 2.7 us a
 // step when every thread has one cell or pair (clock64 of an 8 x 256 lattice: 1300 cycles psi, 930
 // collision, 950 release, 2000 until the neighbours' counts arrive); the redundant psi of the ring is
-// cheap beside it.  Measured a step, two launches -> tiles (us): D2Q9 FP32 8 x 256 8.3 -> 2.7, 256 x 256
-// 8.3 -> 3.6, 512 x 512 10.4 -> 6.5; D3Q19 FP32 32^3 9.3 -> 4.0, 64^3 14.6 -> 10.8; D2Q9 FP64 100 x 100
-// 26.8 -> 18.3, 301 x 203 91 -> 66.
+// cheap beside it.  Microseconds a step, kernels of a single step (which start under the tail of the one
+// before) and tiles, 100 steps a call: D2Q9 FP32 8 x 256 4.3 and 2.6, 256 x 256 5.2 and 3.5, 512 x 512 7.0 and
+// 6.1; D3Q19 FP32 32^3 7.1 and 3.8, 48^3 8.4 and 6.8; D2Q9 FP64 256 x 256 70 and 61, 301 x 203 82 and 58.
 #pragma once
 #include "plb_pair.cuh"
 
