@@ -666,11 +666,12 @@ template <class L, class S> struct Launch {
         if constexpr (Store<S>::SHIFT) {
             if (p.stochastic) {
                 go_long(k_collide_staged<L, S, MRT, ODD, true, WIDE>, grid, sp.threads, st, p, planes(p, A),
-                   (const float *)psi, sp);
+                        (const float *)psi, sp);
                 return;
             }
         }
-        go_long(k_collide_staged<L, S, MRT, ODD, false, WIDE>, grid, sp.threads, st, p, planes(p, A), (const float *)psi, sp);
+        go_long(k_collide_staged<L, S, MRT, ODD, false, WIDE>, grid, sp.threads, st, p, planes(p, A),
+                (const float *)psi, sp);
     }
     template <int MRT, bool ODD> static void collide_t(const KParams &p, void *A, const void *psi, cudaStream_t st) {
         dim3 grid, block;
@@ -786,10 +787,11 @@ template <class L, class S> struct Launch {
         }
         return nb;
     }
-    // single pass: tiles of FusedTile's size, each block walking a chunk of zc planes.  The chunk count minimises (waves of resident blocks) x (planes per chunk + 0.5): a block also forms
-    // psi of the two planes before its chunk, at about a third of a collided plane's cost each
-    // (measured with tiles of 64 x 16 and kept for 64 x 8),
-    // and the last wave of a grid that is not a multiple of the resident blocks runs partly idle.
+    // single pass: tiles of FusedTile's size, each block walking a chunk of zc planes.  The chunk count
+    // minimises (waves of resident blocks) x (planes per chunk + 0.5): a block also forms psi of the two
+    // planes before its chunk, at about a third of a collided plane's cost each (measured with tiles of
+    // 64 x 16 and kept for 64 x 8), and the last wave of a grid that is not a multiple of the resident
+    // blocks runs partly idle.
     template <int MRT> static void fused_t(const KParams &p, const void *A, void *B, cudaStream_t st) {
         if constexpr (!std::is_same<S, double>::value) {
             using Tl = FusedTile<L, S>;
@@ -878,7 +880,9 @@ template <class L, class S> struct Launch {
         const int nw = p.nx / w, sms = sm_count();
         constexpr bool d3 = L::D == 3, fp64 = std::is_same<S, double>::value, fp32 = std::is_same<S, float>::value;
         const long long most_cells = fp64 ? (d3 ? 1 << 14 : 10 << 14)
-                                   : FORM || !d3 ? 1 << 18 : fp32 ? (w == 2 ? 14 << 14 : 7 << 14) : (w == 2 ? 1 << 18 : 1 << 17);
+                                   : FORM || !d3 ? 1 << 18
+                                   : fp32        ? (w == 2 ? 14 << 14 : 7 << 14)
+                                                 : (w == 2 ? 1 << 18 : 1 << 17);
         if (p.n > most_cells) return false;
         const long long work = p.n * (2 / w);
         t.least = FORM || fp64 || (d3 && !fp32 && w == 2) || work <= 1 << 16 ? 2

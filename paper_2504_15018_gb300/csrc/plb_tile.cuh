@@ -80,6 +80,7 @@ __global__ void __maxnreg__((TileThreads<L, S>::regs)) k_tile(KParams p, TileArg
     int2 *cells = reinterpret_cast<int2 *>(psi + (size_t)W * t.max_region);
     int *mine = reinterpret_cast<int *>(cells + t.max_region);
     const int sy = W * (tw + 2), sz = sy * (th + 2);
+    const unsigned gave_up = ld_relaxed(t.counts);                 // (here, under the set-up)
     for (int r = tid; r < region; r += blockDim.x) {
         const int lx = r % (tw + 2), ly = (r / (tw + 2)) % (th + 2), lz = r / ((tw + 2) * (th + 2));
         const bool in = lx >= 1 && lx <= tw && ly >= 1 && ly <= th && lz >= zr && lz < td + zr;
@@ -116,7 +117,7 @@ __global__ void __maxnreg__((TileThreads<L, S>::regs)) k_tile(KParams p, TileArg
     const unsigned start = *reinterpret_cast<volatile unsigned *>(count);
     S *src = static_cast<S *>(t.a), *dst = static_cast<S *>(t.b);
     for (int s = 0; s < t.nsteps; ++s) {
-        int ok = s > 0 || ld_relaxed(t.counts) == 0;
+        int ok = s > 0 || gave_up == 0;
         if (s > 0 && watch) {
             unsigned spins = 0;
             while ((int)(ld_relaxed(watch) - (start + (unsigned)s)) < 0) {
